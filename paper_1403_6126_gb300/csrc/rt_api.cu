@@ -111,6 +111,7 @@ rtg::StepArgs<Real> rtg::make_args(rt_ctx *c, double dt) {
   a.kv_per_rho = c->opt.r_ideal / (c->opt.gamma - 1.0);
   a.hold_T = c->opt.hold_T;
   a.estimate_v = c->opt.estimate_v;
+  a.sym = c->sym;
   a.newton_max_it = c->opt.newton_max_it;
   a.newton_rtol = c->opt.newton_rtol;
   a.wnorm = (Real)rtg::weight_norm(c->host_angf.data(), c->M);
@@ -161,6 +162,7 @@ cudaError_t rtg::launch_ctx_step_on(rt_ctx *c, const StepArgs<double> &a, bool v
 
 cudaError_t rtg::launch_ctx_step_on(rt_ctx *c, const StepArgs<float> &a, bool vel, TileShape t, cudaStream_t s) {
   if (c->bf16) return launch_step<float>(a, c->dim, vel, t, s);
+  if (c->sym) return launch_step_sym(a, c->host_angf.data(), c->host_inflowf.data(), c->dim, vel, t, s);
   return launch_step_quad(a, c->host_angf.data(), c->host_inflowf.data(), c->dim, vel, t, s);
 }
 
@@ -441,6 +443,14 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
     for (int d = 0; d < 3; ++d) c->host_angf[4 * m + d] = (float)ang->n[3 * m + d];
     c->host_angf[4 * m + 3] = (float)ang->w[m];
   }
+  c->order.resize(M);
+  c->sym = c->quad && c->dim >= 2 && rtg::pair_order(c->host_angf.data(), M, c->order.data());
+  for (int i = 0; i < M; ++i) {
+    if (!c->sym) c->order[i] = i;
+    c->map.slot[c->order[i]] = (unsigned char)i;
+    for (int d = 0; d < 3; ++d) c->host_angf[4 * i + d] = (float)ang->n[3 * c->order[i] + d];
+    c->host_angf[4 * i + 3] = (float)ang->w[c->order[i]];
+  }
   c->host_inflowf.assign(6 * (size_t)M, 0.0f);
   bool ok = c->fp64 ? rtg::choose_tile<double>(c->dim, M, true, &c->tile)
             : c->bf16 ? rtg::choose_tile_b16(c->dim, M, &c->tile)
@@ -477,9 +487,10 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
   }
   // angle table [M][4] = (n_x, n_y, n_z, W) and zero inflow, via the stage
   std::vector<double> tab(4 * (size_t)M);
-  for (int m = 0; m < M; ++m) {
-    for (int d = 0; d < 3; ++d) tab[4 * m + d] = ang->n[3 * m + d];
-    tab[4 * m + 3] = ang->w[m];
+  for (int i = 0; i < M; ++i) {
+    const int m = c->order[i];
+    for (int d = 0; d < 3; ++d) tab[4 * i + d] = ang->n[3 * m + d];
+    tab[4 * i + 3] = ang->w[m];
   }
   rt_status st = RT_OK;
   cudaError_t e = cudaMemcpyAsync(c->stage, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream);
@@ -562,7 +573,7 @@ rt_status rt_set_intensity(rt_ctx *c, const double *I) {
       rt_status st = fetch(c, I + off, c->stage, n);
       if (st != RT_OK) return st;
       if (c->quad) {
-        RT_CUDA(rtg::launch_quad_in(c->stage, (float *)dst, off, n, N, c->stream));
+        RT_CUDA(rtg::launch_quad_in(c->stage, (float *)dst, off, n, N, c->map, c->stream));
       } else {
         st = convert_in(c, c->stage, (char *)dst + off * rsd, n);
         if (st != RT_OK) return st;
@@ -580,17 +591,39 @@ rt_status rt_set_intensity(rt_ctx *c, const double *I) {
   return RT_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The float host table and the device table (stored order) from host_inflow.
+// Waits for the stream.
+rt_status inflow_tables(rt_ctx *c) {
+  const int M = c->M;
+  std::vector<double> in(6 * (size_t)M);
+  for (int f = 0; f < 6; ++f)
+    for (int i = 0; i < M; ++i) {
+      in[(size_t)f * M + i] = c->host_inflow[(size_t)f * M + c->order[i]];
+      c->host_inflowf[(size_t)f * M + i] = (float)in[(size_t)f * M + i];
+    }
+  RT_CUDA(cudaMemcpyAsync(c->stage, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  rt_status st = convert_in(c, c->stage, c->inflow, 6 * M);
+  if (st != RT_OK) return st;
+  RT_CUDA(cudaStreamSynchronize(c->stream));
+  return RT_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 rt_status rt_set_inflow(rt_ctx *c, int axis, int side, const double *I_ghost) {
   if (!c || !I_ghost) return fail(RT_E_INVALID, "rt_set_inflow: NULL argument");
   if (axis < 0 || axis >= c->dim || side < 0 || side > 1) return fail(RT_E_INVALID, "rt_set_inflow: bad face");
   for (int m = 0; m < c->M; ++m)
     if (!std::isfinite(I_ghost[m]) || I_ghost[m] < 0) return fail(RT_E_NONFINITE, "rt_set_inflow: need finite I >= 0");
   std::copy(I_ghost, I_ghost + c->M, c->host_inflow.begin() + (size_t)(axis * 2 + side) * c->M);
-  for (int m = 0; m < c->M; ++m) c->host_inflowf[(size_t)(axis * 2 + side) * c->M + m] = (float)I_ghost[m];
-  RT_CUDA(cudaMemcpyAsync(c->stage, c->host_inflow.data(), 6 * c->M * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  rt_status st = convert_in(c, c->stage, c->inflow, 6 * c->M);
+  rt_status st = inflow_tables(c);
   if (st != RT_OK) return st;
-  RT_CUDA(cudaStreamSynchronize(c->stream));
   // the float step carries the table in its launch parameters: a graph
   // captured by rt_run holds the old one
   if (c->graph) {
@@ -764,10 +797,26 @@ rt_status rt_save_state(rt_ctx *c, void *buf, size_t bytes) {
   size_t b[16];
   const int k = state_parts(c, p, b);
   for (int i = 0; i < k; ++i) {
-    RT_CUDA(cudaMemcpyAsync(out, p[i], b[i], cudaMemcpyDeviceToHost, c->stream));
+    if (c->sym && i == 0) {
+      // the state holds the intensity in the caller's order of the angles
+      const size_t plane = sizeof(float4) * (size_t)c->N;
+      for (int q = 0; q < c->M / 4; ++q) {
+        RT_CUDA(rtg::launch_plane_out((const float *)p[i], (float *)c->stage, q, c->N, c->map, c->stream));
+        RT_CUDA(cudaMemcpyAsync(out + q * plane, c->stage, plane, cudaMemcpyDeviceToHost, c->stream));
+      }
+    } else {
+      RT_CUDA(cudaMemcpyAsync(out, p[i], b[i], cudaMemcpyDeviceToHost, c->stream));
+    }
     out += b[i];
   }
   RT_CUDA(cudaStreamSynchronize(c->stream));
+  if (c->sym) {   // the last part, the inflow table, too
+    float *t = reinterpret_cast<float *>(out - b[k - 1]);
+    for (size_t i = 0; i < 6 * (size_t)c->M; ++i) {
+      const float v = (float)c->host_inflow[i];
+      std::memcpy(t + i, &v, sizeof v);
+    }
+  }
   return RT_OK;
 }
 
@@ -787,17 +836,25 @@ rt_status rt_load_state(rt_ctx *c, const void *buf, size_t bytes) {
   c->cur = 0;
   const char *in = static_cast<const char *>(buf) + sizeof h;
   std::memcpy(c->host_inflow.data(), in, sizeof(double) * 6 * (size_t)c->M);
-  // the float step takes its inflow from the host's float table (launch
-  // parameters), the batch kernel from the device table restored below
-  for (size_t i = 0; i < 6 * (size_t)c->M; ++i) c->host_inflowf[i] = (float)c->host_inflow[i];
   in += sizeof(double) * 6 * (size_t)c->M;
   void *p[16];
   size_t b[16];
   const int k = state_parts(c, p, b);
   for (int i = 0; i < k; ++i) {
-    RT_CUDA(cudaMemcpyAsync(p[i], in, b[i], cudaMemcpyHostToDevice, c->stream));
+    if (c->sym && i == 0) {
+      const size_t plane = sizeof(float4) * (size_t)c->N;
+      for (int q = 0; q < c->M / 4; ++q) {
+        RT_CUDA(cudaMemcpyAsync(c->stage, in + q * plane, plane, cudaMemcpyHostToDevice, c->stream));
+        RT_CUDA(rtg::launch_plane_in((const float *)c->stage, (float *)p[i], q, c->N, c->map, c->stream));
+      }
+    } else {
+      RT_CUDA(cudaMemcpyAsync(p[i], in, b[i], cudaMemcpyHostToDevice, c->stream));
+    }
     in += b[i];
   }
+  // the float step takes its inflow from the host's float table (launch
+  // parameters), the batch kernel from the device table
+  if (rt_status st = inflow_tables(c); st != RT_OK) return st;
   RT_CUDA(cudaMemsetAsync(c->flags, 0, 2 * sizeof(int), c->stream));
   // the float step's cell centers are a function of the intensity: formed
   // again rather than saved
@@ -1063,7 +1120,7 @@ rt_status rt_get_intensity(rt_ctx *c, double *I) {
                                              c->N, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "decode");
     } else if (c->quad) {
-      cudaError_t e = rtg::launch_quad_out((const float *)c->I[c->cur], c->stage, off, n, c->N, c->stream);
+      cudaError_t e = rtg::launch_quad_out((const float *)c->I[c->cur], c->stage, off, n, c->N, c->map, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "quad layout");
     } else {
       st = convert_out(c, (const char *)c->I[c->cur] + off * c->rs, c->stage, n);

@@ -62,21 +62,48 @@ __global__ void isotropic_quad_kernel(const double *__restrict__ T, float4 *__re
 }
 
 // Angle-major doubles, elements [off, off + n) (element i: angle i / N of
-// cell i % N), into the quad layout (element (m, c) at float (m/4) 4N + 4c
-// + m%4), and back.
+// cell i % N), into the quad layout (angle m of cell c at float (s/4) 4N + 4c
+// + s%4, s = map.slot[m]), and back.
 __global__ void quad_in_kernel(const double *__restrict__ src, float *__restrict__ dst, long long off, long long n,
-                               long long N) {
+                               long long N, const AngleMap map) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long g = off + i, m = g / N, c = g - m * N;
-    dst[(m >> 2) * 4 * N + 4 * c + (m & 3)] = (float)src[i];
+    const long long g = off + i, m = g / N, c = g - m * N, k = map.slot[m];
+    dst[(k >> 2) * 4 * N + 4 * c + (k & 3)] = (float)src[i];
   }
 }
 
 __global__ void quad_out_kernel(const float *__restrict__ src, double *__restrict__ dst, long long off, long long n,
-                                long long N) {
+                                long long N, const AngleMap map) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long g = off + i, m = g / N, c = g - m * N;
-    dst[i] = (double)src[(m >> 2) * 4 * N + 4 * c + (m & 3)];
+    const long long g = off + i, m = g / N, c = g - m * N, k = map.slot[m];
+    dst[i] = (double)src[(k >> 2) * 4 * N + 4 * c + (k & 3)];
+  }
+}
+
+// The caller's angles 4q .. 4q + 3 of every cell as one float4 plane.
+__global__ void plane_out_kernel(const float *__restrict__ I, float4 *__restrict__ dst, int q, long long N,
+                                 const AngleMap map) {
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
+    float v[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const long long k = map.slot[4 * q + h];
+      v[h] = I[(k >> 2) * 4 * N + 4 * c + (k & 3)];
+    }
+    dst[c] = make_float4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+__global__ void plane_in_kernel(const float4 *__restrict__ src, float *__restrict__ I, int q, long long N,
+                                const AngleMap map) {
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
+    const float4 x = src[c];
+    const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const long long k = map.slot[4 * q + h];
+      I[(k >> 2) * 4 * N + 4 * c + (k & 3)] = v[h];
+    }
   }
 }
 
@@ -314,15 +341,27 @@ cudaError_t launch_eddington(const double *mom, double *f, long long N, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t launch_quad_in(const double *src, float *dst, long long off, long long n, long long N, cudaStream_t s) {
+cudaError_t launch_quad_in(const double *src, float *dst, long long off, long long n, long long N, const AngleMap &map,
+                           cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  quad_in_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, dst, off, n, N);
+  quad_in_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, dst, off, n, N, map);
   return cudaGetLastError();
 }
 
-cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, cudaStream_t s) {
+cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, const AngleMap &map,
+                            cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  quad_out_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, dst, off, n, N);
+  quad_out_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, dst, off, n, N, map);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plane_out(const float *I, float *dst, int q, long long N, const AngleMap &map, cudaStream_t s) {
+  plane_out_kernel<<<grid_for(N, 256), 256, 0, s>>>(I, reinterpret_cast<float4 *>(dst), q, N, map);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plane_in(const float *src, float *I, int q, long long N, const AngleMap &map, cudaStream_t s) {
+  plane_in_kernel<<<grid_for(N, 256), 256, 0, s>>>(reinterpret_cast<const float4 *>(src), I, q, N, map);
   return cudaGetLastError();
 }
 

@@ -85,23 +85,18 @@ rt_status rebuild(rt_batch *b) {
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->ctxs[x]->M > b->ctxs[y]->M; });
   const rtg::BatchVariant &var = rtg::batch_variant(b->variant);
   std::vector<rtg::WorkItem> items;
-  int Mmax = 1;
-  bool dims[4] = {false, false, false, false};
+  size_t smem = 0;
   b->vel = false;
   for (rt_ctx *c : b->ctxs) b->vel = b->vel || rtg::velocity_on(c);
   for (int i : order) {
     rt_ctx *c = b->ctxs[i];
-    Mmax = std::max(Mmax, c->M);
-    dims[c->dim] = true;
+    smem = std::max(smem, c->sym ? var.smem_sym(c->dim, b->vel) : rtg::variant_smem(var, c->dim, c->M, b->vel));
     const rtg::TileShape t = c->dim == 1 ? var.t1 : c->dim == 2 ? var.t2 : var.t3;
     const int tx = t.tx, ty = t.ty, tz = t.tz;
     for (int z = 0; z < (c->n[2] + tz - 1) / tz; ++z)
       for (int y = 0; y < (c->n[1] + ty - 1) / ty; ++y)
         for (int x = 0; x < (c->n[0] + tx - 1) / tx; ++x) items.push_back({i, x, y, z});
   }
-  size_t smem = 0;
-  for (int d = 1; d <= 3; ++d)
-    if (dims[d]) smem = std::max(smem, rtg::variant_smem(var, d, Mmax, b->vel));
   if (smem > 227 * 1024)
     return rtg::set_error(RT_E_INVALID, "rt_batch: the largest angle set does not fit the batch tile in shared memory");
   b->smem = smem;

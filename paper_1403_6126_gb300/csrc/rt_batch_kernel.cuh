@@ -4,7 +4,7 @@
 // tile set; all shapes of a set have the same thread count (one per cell).
 #pragma once
 
-#include "rt_step_quad.cuh"
+#include "rt_step_sym.cuh"
 
 namespace rtg {
 
@@ -16,6 +16,7 @@ struct WorkItem {
 struct BatchVariant {
   int threads;
   TileShape t1, t2, t3;   // tiles of 1-D, 2-D and 3-D members
+  size_t (*smem_sym)(int dim, bool vel);   // of a member stored as opposite pairs
   cudaError_t (*prepare)(bool vel, size_t smem, int *blocks_per_sm);
   cudaError_t (*launch)(bool vel, int grid, size_t smem, const StepArgs<float> *descs, const WorkItem *items,
                         int nitems, cudaStream_t s);
@@ -46,7 +47,11 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       __syncthreads();
       cur = w.prob;
     }
-    if (desc.dim == 3)
+    if (desc.sym && desc.dim == 3)
+      stepk::process_tile_sym<3, VEL, X3, Y3, Z3, false, false>(desc, nullptr, tid, w.tbx, w.tby, w.tbz, smem);
+    else if (desc.sym)
+      stepk::process_tile_sym<2, VEL, X2, Y2, 1, false, false>(desc, nullptr, tid, w.tbx, w.tby, 0, smem);
+    else if (desc.dim == 3)
       stepk::process_tile_q<3, VEL, X3, Y3, Z3, false, 2>(desc, nullptr, tid, w.tbx, w.tby, w.tbz, smem);
     else if (desc.dim == 2)
       stepk::process_tile_q<2, VEL, X2, Y2, 1, false, 2>(desc, nullptr, tid, w.tbx, w.tby, 0, smem);
@@ -57,6 +62,11 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 
 template <int NT, int X2, int Y2, int X3, int Y3, int Z3>
 struct BatchImpl {
+  static size_t smem_sym(int dim, bool vel) {
+    if (dim == 3)
+      return vel ? stepk::smem_bytes_sym_t<3, true, X3, Y3, Z3>(false) : stepk::smem_bytes_sym_t<3, false, X3, Y3, Z3>(false);
+    return vel ? stepk::smem_bytes_sym_t<2, true, X2, Y2, 1>(false) : stepk::smem_bytes_sym_t<2, false, X2, Y2, 1>(false);
+  }
   static cudaError_t prepare(bool vel, size_t smem, int *per_sm) {
     auto kern = vel ? batch_kernel<true, NT, X2, Y2, X3, Y3, Z3> : batch_kernel<false, NT, X2, Y2, X3, Y3, Z3>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -70,7 +80,7 @@ struct BatchImpl {
     return cudaGetLastError();
   }
   static BatchVariant describe() {
-    return BatchVariant{NT, TileShape{NT, 1, 1}, TileShape{X2, Y2, 1}, TileShape{X3, Y3, Z3}, &prepare, &launch};
+    return BatchVariant{NT, TileShape{NT, 1, 1}, TileShape{X2, Y2, 1}, TileShape{X3, Y3, Z3}, &smem_sym, &prepare, &launch};
   }
 };
 

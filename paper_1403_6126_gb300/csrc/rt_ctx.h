@@ -22,6 +22,9 @@ struct rt_ctx {
   size_t rs = 4;      // bytes per stored real of the cell data (rho, sigma, v)
   size_t rsI = 4;     // bytes per stored intensity
   bool quad = false;  // float intensities in the quad-interleaved layout (RT_FP32)
+  bool sym = false;   // its angles stored as opposite pairs (rtg::pair_order)
+  std::vector<int> order;  // the caller's index of each stored angle (identity unless sym)
+  rtg::AngleMap map{};     // and where each of the caller's angles is stored
   size_t I_bytes = 0; // bytes of one intensity buffer
   float *qscr = nullptr;  // bf16 storage: float [M][N] scratch for Q_m
   float *cen[2] = {nullptr, nullptr};   // float step: each cell's smallest intensity over angles [N]
@@ -39,8 +42,9 @@ struct rt_ctx {
   double *stage = nullptr;
   long long stage_len = 0;
   std::vector<double> host_n, host_w, host_inflow;
-  // the angle table [M][4] and inflow table [6][M] rounded to float, as the
-  // device tables hold them (launch-parameter tables of the float kernel)
+  // the angle table [M][4] and inflow table [6][M] rounded to float, in stored
+  // order, as the device tables hold them (launch-parameter tables of the
+  // float kernels); host_n, host_w, host_inflow are in the caller's order
   std::vector<float> host_angf, host_inflowf;
   // captured multi-step graph
   cudaGraphExec_t graph = nullptr;

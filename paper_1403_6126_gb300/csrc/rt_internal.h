@@ -31,6 +31,7 @@ struct StepArgs {
   float msum[10][2];  // the float table's normalised quadrature sums (table_moment_sums)
   const Real *ang;    // [M][4]: n_x, n_y, n_z, W
   const Real *inflow; // [3][2][M]
+  int sym;            // float quad layout: angles stored as opposite pairs (pair_order)
   // Intensities.  Double: angle-major [M][N].  Float: quad-interleaved,
   // ceil(M/4) planes of float4 ([q][c] holds angles 4q .. 4q+3 of cell c,
   // angles past M zero).
@@ -134,6 +135,23 @@ bool choose_tile_b16(int dim, int M, TileShape *out);
 cudaError_t launch_step_quad(const StepArgs<float> &a, const float *host_ang, const float *host_inflow, int dim,
                              bool vel, TileShape t, cudaStream_t s);
 
+// Opposite pairs (rt_step_sym.cuh): whether the angles of a float table ang4
+// ([M][4]: n_x, n_y, n_z, W) are pairs (n, -n) of one weight, exactly as the
+// floats stand (those of every level-symmetric set are), whole quads of them
+// and at most 80 angles.  Then order[i] is the index of the angle stored i-th.
+bool pair_order(const float *ang4, int M, int *order);
+
+// The float step on opposite pairs: host_ang, host_inflow and the intensities
+// in stored order.
+cudaError_t launch_step_sym(const StepArgs<float> &a, const float *host_ang, const float *host_inflow, int dim,
+                            bool vel, TileShape t, cudaStream_t s);
+
+// Where each of the caller's angles is stored (identity unless the set is
+// stored as opposite pairs).
+struct AngleMap {
+  unsigned char slot[kMaxAngles];
+};
+
 // Elementwise helpers (all stream-ordered).
 template <typename Real>
 cudaError_t launch_convert_in(const double *src, Real *dst, long long n, cudaStream_t s);
@@ -155,8 +173,14 @@ cudaError_t launch_centers(const float *I, int M, long long N, float *cen, cudaS
 cudaError_t launch_eddington(const double *mom, double *f, long long N, cudaStream_t s);
 // Elements [off, off + n) of an angle-major double field (element i is angle
 // i / N of cell i % N) into / out of the quad-interleaved float layout.
-cudaError_t launch_quad_in(const double *src, float *dst, long long off, long long n, long long N, cudaStream_t s);
-cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, cudaStream_t s);
+cudaError_t launch_quad_in(const double *src, float *dst, long long off, long long n, long long N, const AngleMap &map,
+                           cudaStream_t s);
+cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, const AngleMap &map,
+                            cudaStream_t s);
+// One plane of four angles (the caller's 4q .. 4q + 3) of an array stored
+// through map, as float4 per cell: out of I into dst, or (in) from src into I.
+cudaError_t launch_plane_out(const float *I, float *dst, int q, long long N, const AngleMap &map, cudaStream_t s);
+cudaError_t launch_plane_in(const float *src, float *I, int q, long long N, const AngleMap &map, cudaStream_t s);
 
 // bf16 storage: encode a float intensity array [M][N] as deviations from
 // the mean intensity of each cell (E [N] its energy density), and decode

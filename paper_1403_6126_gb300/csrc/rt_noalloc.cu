@@ -22,7 +22,7 @@
 
 #include "rt.h"
 #include "rt_ctx.h"
-#include "rt_step_quad.cuh"
+#include "rt_step_sym.cuh"
 
 namespace rtg {
 
@@ -50,13 +50,26 @@ __global__ void __launch_bounds__(TX * TY * TZ, stepk::kQMinBlocks<TX * TY * TZ>
         a, &qt, threadIdx.x, it % ntx, (it / ntx) % nty, it / (ntx * nty), smem);
 }
 
+// The same for a set of opposite pairs: read and written in the caller's order
+// of the angles, computed in the stored order of a context.
+template <int DIM, int TX, int TY, int TZ>
+__global__ void __launch_bounds__(TX * TY * TZ, stepk::kQMinBlocks<TX * TY * TZ>)
+    noalloc_kernel_sym(const StepArgs<float> a, const __grid_constant__ stepk::SymTable tab) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int ntx = (a.n[0] + TX - 1) / TX, nty = (a.n[1] + TY - 1) / TY, ntz = (a.n[2] + TZ - 1) / TZ;
+  const int ntiles = ntx * nty * ntz;
+  for (int it = blockIdx.x; it < ntiles; it += gridDim.x)
+    stepk::process_tile_sym<DIM, true, TX, TY, TZ, true, true>(a, &tab, threadIdx.x, it % ntx, (it / ntx) % nty,
+                                                               it / (ntx * nty), smem);
+}
+
 // Per device: the scratch array's device address, and per dimension the SM
 // count and resident CTAs at the shared-memory size last set.
 struct DeviceCache {
   void *scratch = nullptr;
   int sms = 0;
-  size_t smem[3] = {0, 0, 0};
-  int per_sm[3] = {0, 0, 0};
+  size_t smem[5] = {0, 0, 0, 0, 0};   // per kernel: 1-D, 2-D, 3-D; 2-D, 3-D on opposite pairs
+  int per_sm[5] = {0, 0, 0, 0, 0};
 };
 struct NoallocState {
   std::mutex mu;
@@ -92,29 +105,42 @@ rt_status scratch_for(int dev, unsigned char **out) {
   return RT_OK;
 }
 
-template <int DIM, int TX, int TY, int TZ>
-cudaError_t launch_noalloc(const StepArgs<float> &a, const NoallocTable &qt, int dev, cudaStream_t s) {
-  const size_t sm = stepk::smem_bytes_q(DIM, a.M, true, TX, TY, TZ, true);
-  auto kern = noalloc_kernel<DIM, TX, TY, TZ>;
+// Launches kern (cache entry k) with the launch-parameter table t and sm bytes
+// of shared memory.
+template <int TX, int TY, int TZ, class Kern, class Table>
+cudaError_t launch_noalloc(Kern kern, int k, const StepArgs<float> &a, const Table &t, size_t sm, int dev,
+                           cudaStream_t s) {
   int per_sm = 0, sms = 0;
   {
     // the attribute and the occupancy are set / asked only when the shared
-    // memory grows past what this device's kernel of this dimension has seen
+    // memory grows past what this device's kernel has seen
     std::lock_guard<std::mutex> lock(g_state.mu);
     DeviceCache &d = g_state.dev[dev];
-    if (sm > d.smem[DIM - 1]) {
+    if (sm > d.smem[k]) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.per_sm[DIM - 1], kern, TX * TY * TZ, sm);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.per_sm[k], kern, TX * TY * TZ, sm);
       if (e != cudaSuccess) return e;
-      d.smem[DIM - 1] = sm;
+      d.smem[k] = sm;
     }
-    per_sm = std::max(1, d.per_sm[DIM - 1]);
+    per_sm = std::max(1, d.per_sm[k]);
     sms = d.sms;
   }
   const long long ntiles = (long long)((a.n[0] + TX - 1) / TX) * ((a.n[1] + TY - 1) / TY) * ((a.n[2] + TZ - 1) / TZ);
   const int grid = (int)std::max(1LL, std::min(ntiles, (long long)sms * per_sm));
-  kern<<<grid, TX * TY * TZ, sm, s>>>(a, qt);
+  kern<<<grid, TX * TY * TZ, sm, s>>>(a, t);
   return cudaGetLastError();
+}
+
+template <int DIM, int TX, int TY, int TZ>
+cudaError_t launch_noalloc_quad(const StepArgs<float> &a, const NoallocTable &qt, int dev, cudaStream_t s) {
+  return launch_noalloc<TX, TY, TZ>(noalloc_kernel<DIM, TX, TY, TZ>, DIM - 1, a, qt,
+                                    stepk::smem_bytes_q(DIM, a.M, true, TX, TY, TZ, true), dev, s);
+}
+
+template <int DIM, int TX, int TY, int TZ>
+cudaError_t launch_noalloc_sym(const StepArgs<float> &a, const stepk::SymTable &tab, int dev, cudaStream_t s) {
+  return launch_noalloc<TX, TY, TZ>(noalloc_kernel_sym<DIM, TX, TY, TZ>, DIM + 1, a, tab,
+                                    stepk::smem_bytes_gather_t<DIM, true, TX, TY, TZ>(a.M), dev, s);
 }
 
 }  // namespace
@@ -189,13 +215,23 @@ extern "C" rt_status rt_step_noalloc(const rt_grid *g, const rt_angles *ang, dou
   if ((st = rtg::scratch_for(dev, &scratch)) != RT_OK) return st;
   int *counter = reinterpret_cast<int *>(scratch);
 
-  // the angle table as the device would round it, and the inflow table
+  // the angle table as the device would round it, and the inflow table, in
+  // the order a context would store them
   float angf[4 * rtg::kNoallocMaxAngles], inflowf[6 * rtg::kNoallocMaxAngles];
   for (int m = 0; m < M; ++m) {
     for (int d = 0; d < 3; ++d) angf[4 * m + d] = (float)ang->n[3 * m + d];
     angf[4 * m + 3] = (float)ang->w[m];
   }
-  for (int i = 0; i < 6 * M; ++i) inflowf[i] = f->inflow ? (float)f->inflow[i] : 0.0f;
+  int order[rtg::kNoallocMaxAngles];
+  const bool sym = g->dim >= 2 && rtg::pair_order(angf, M, order);
+  if (sym)
+    for (int i = 0; i < M; ++i) {
+      for (int d = 0; d < 3; ++d) angf[4 * i + d] = (float)ang->n[3 * order[i] + d];
+      angf[4 * i + 3] = (float)ang->w[order[i]];
+    }
+  for (int k = 0; k < 6; ++k)
+    for (int i = 0; i < M; ++i) inflowf[k * M + i] = f->inflow ? (float)f->inflow[k * M + (sym ? order[i] : i)] : 0.0f;
+  a.sym = sym;
   a.M = M;
   a.N = N;
   a.C = (float)Crat;
@@ -232,14 +268,21 @@ extern "C" rt_status rt_step_noalloc(const rt_grid *g, const rt_angles *ang, dou
   a.Q = nullptr;
   a.outer_begin = 0;
   a.outer_count = 0;
-  rtg::NoallocTable qt;   // 22 KB, passed by value as the launch parameters
-  rtg::stepk::fill_qtable(&qt, angf, M, a.C, a.dtdx, inflowf);
-
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), s);   // the failure word
   if (e != cudaSuccess) return set_error(RT_E_CUDA, std::string("rt_step_noalloc: clear: ") + cudaGetErrorString(e));
-  e = g->dim == 1   ? rtg::launch_noalloc<1, 512, 1, 1>(a, qt, dev, s)
-      : g->dim == 2 ? rtg::launch_noalloc<2, 32, 16, 1>(a, qt, dev, s)
-                    : rtg::launch_noalloc<3, 8, 8, 4>(a, qt, dev, s);
+  // the tables travel by value as launch parameters
+  if (sym) {
+    rtg::stepk::SymTable tab;
+    rtg::stepk::fill_symtable(&tab, angf, M, a.C, a.dtdx, inflowf, order);
+    e = g->dim == 2 ? rtg::launch_noalloc_sym<2, 32, 16, 1>(a, tab, dev, s)
+                    : rtg::launch_noalloc_sym<3, 8, 8, 4>(a, tab, dev, s);
+  } else {
+    rtg::NoallocTable qt;   // 22 KB
+    rtg::stepk::fill_qtable(&qt, angf, M, a.C, a.dtdx, inflowf);
+    e = g->dim == 1   ? rtg::launch_noalloc_quad<1, 512, 1, 1>(a, qt, dev, s)
+        : g->dim == 2 ? rtg::launch_noalloc_quad<2, 32, 16, 1>(a, qt, dev, s)
+                      : rtg::launch_noalloc_quad<3, 8, 8, 4>(a, qt, dev, s);
+  }
   if (e != cudaSuccess) return set_error(RT_E_CUDA, std::string("rt_step_noalloc: launch: ") + cudaGetErrorString(e));
   if (newton_failures) {
     e = cudaMemcpyAsync(newton_failures, counter, sizeof(int), cudaMemcpyDeviceToHost, s);

@@ -20,6 +20,7 @@ namespace rtg {
 namespace stepk {
 template <int P>
 struct QTable;
+struct SymTable;
 }
 // Launchers of the compiled shapes, one translation unit per group; they
 // return cudaErrorInvalidConfiguration for a shape that is not compiled.
@@ -28,5 +29,8 @@ struct QTable;
 cudaError_t launch_f3(const StepArgs<float> &a, const stepk::QTable<40> *qt, bool vel, TileShape t, cudaStream_t s);
 cudaError_t launch_f12(const StepArgs<float> &a, const stepk::QTable<40> *qt, int dim, bool vel, TileShape t,
                        cudaStream_t s);
+// The pair kernel's shapes (rt_step_sym.cuh).
+cudaError_t launch_s3(const StepArgs<float> &a, const stepk::SymTable &tab, bool vel, TileShape t, cudaStream_t s);
+cudaError_t launch_s2(const StepArgs<float> &a, const stepk::SymTable &tab, bool vel, TileShape t, cudaStream_t s);
 cudaError_t launch_d(const StepArgs<double> &a, int dim, bool vel, TileShape t, cudaStream_t s);
 }  // namespace rtg

@@ -1,9 +1,9 @@
-// Tile choice and dispatch of the fused step kernels (rt_step_quad.cuh for
-// float intensities, rt_step_pair.cuh for their bf16 storage,
+// Tile choice and dispatch of the fused step kernels (rt_step_sym.cuh and
+// rt_step_quad.cuh for float intensities, rt_step_pair.cuh for their bf16 storage,
 // rt_step_kernel.cuh for double): the compiled shapes are listed in
 // rt_shapes.h.
 #include "rt_shapes.h"
-#include "rt_step_quad.cuh"
+#include "rt_step_sym.cuh"
 
 namespace rtg {
 
@@ -91,6 +91,35 @@ cudaError_t launch_step_quad(const StepArgs<float> &a, const float *host_ang, co
     return dim == 3 ? launch_f3(a, &qt, vel, t, s) : launch_f12(a, &qt, dim, vel, t, s);
   }
   return dim == 3 ? launch_f3(a, nullptr, vel, t, s) : launch_f12(a, nullptr, dim, vel, t, s);
+}
+
+bool pair_order(const float *ang4, int M, int *order) {
+  if (M % 4 != 0 || M > stepk::kSymMaxAngles) return false;
+  bool used[stepk::kSymMaxAngles] = {};
+  int k = 0;
+  for (int m = 0; m < M; ++m) {
+    if (used[m]) continue;
+    const float *n = ang4 + 4 * m;
+    int at = -1;
+    for (int l = m + 1; l < M && at < 0; ++l) {
+      const float *p = ang4 + 4 * l;
+      if (!used[l] && p[0] == -n[0] && p[1] == -n[1] && p[2] == -n[2] && p[3] == n[3]) at = l;
+    }
+    if (at < 0) return false;
+    // quads (n, n', -n, -n')
+    used[m] = used[at] = true;
+    order[k] = m;
+    order[k + 2] = at;
+    k += k % 4 == 0 ? 1 : 3;
+  }
+  return true;
+}
+
+cudaError_t launch_step_sym(const StepArgs<float> &a, const float *host_ang, const float *host_inflow, int dim,
+                            bool vel, TileShape t, cudaStream_t s) {
+  stepk::SymTable tab;
+  stepk::fill_symtable(&tab, host_ang, a.M, a.C, a.dtdx, host_inflow, nullptr);
+  return dim == 3 ? launch_s3(a, tab, vel, t, s) : launch_s2(a, tab, vel, t, s);
 }
 
 template <>

@@ -180,6 +180,228 @@ __device__ __forceinline__ double mom_4pi_double(float R, float sh, float sl, fl
   return ksum_4pi_double(k);
 }
 
+// What the implicit steps of one cell need besides its intensities.
+//
+// Steps 4 and 5 are taken in deviations from the cell's center R (the
+// smallest I^n_m over its angles): every stored right-hand side, every
+// angle sum and both per-cell solves carry quantities of the size of I - R
+// rather than of I, and each per-cell solve is the exact sum of the
+// per-angle updates that follow it.  Float rounding then scales with the
+// spread of the intensities over angle (never above I_m itself, since R
+// <= I_m), and the energy the T^4 solve hands to the gas is the energy
+// the per-angle update takes from the radiation, step after step.
+struct CellIn {
+  float rho, sa, ss, R;
+  float vt[3], vin[3], v2;
+  float A0, A1, kap, a0, a1;   // Step 4: d = A0 - A1 vn; Step 5: a' = a0 - a1 vn
+  float bt0, bt1, bt2;         // beta_m = b_m + a1 C = 2 a1 vn - a1 (v.v + vn^2) / C (b_m of sec. 4.4)
+  float rd0, ra0;              // 1 / A0, 1 / a0 (no velocity terms)
+  double T0;
+  bool to_scat;
+
+  // Everything but R of cell c.
+  template <bool VEL>
+  __device__ __forceinline__ void load(const StepArgs<float> &a, long long c) {
+    const float C = a.C, dt = a.dt;
+    const long long N = a.N;
+    rho = a.rho[c];
+    sa = a.sa[c];
+    ss = a.ss[c];
+    T0 = a.T_in[c];
+    for (int d = 0; d < 3; ++d) vt[d] = vin[d] = 0.0f;
+    if (VEL) {
+      for (int d = 0; d < 3; ++d) vin[d] = a.v[d * N + c];
+      if (a.estimate_v) {
+        const float E = d2f_rn(a.mom_in[c]);
+        const float h = 0.5f * dt * (sa + ss);
+        for (int d = 0; d < 3; ++d) {
+          const float Fd = d2f_rn(a.mom_in[(1 + d) * N + c]), Pdd = d2f_rn(a.mom_in[(4 + d) * N + c]);
+          const float num = rho * vin[d] + h * (C * rho * vin[d] + a.P * Fd);
+          const float den = rho + h * (C * rho + a.P * (E + Pdd) / C);
+          vt[d] = num / den;
+        }
+      } else {
+        vt[0] = vin[0]; vt[1] = vin[1]; vt[2] = vin[2];
+      }
+    }
+    derive<VEL>(a);
+  }
+
+  // The same once v~ and the center are known.
+  template <bool VEL>
+  __device__ __forceinline__ void reload(const StepArgs<float> &a, long long c, const float v_est[3], float center) {
+    rho = a.rho[c];
+    sa = a.sa[c];
+    ss = a.ss[c];
+    T0 = a.T_in[c];
+    R = center;
+    for (int d = 0; d < 3; ++d) {
+      vt[d] = v_est[d];
+      vin[d] = VEL ? a.v[d * a.N + c] : 0.0f;
+    }
+    derive<VEL>(a);
+  }
+
+  template <bool VEL>
+  __device__ __forceinline__ void derive(const StepArgs<float> &a) {
+    const float C = a.C, invC = a.invC, dt = a.dt;
+    to_scat = ss > sa;
+    v2 = vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2];
+    A0 = 1.0f + dt * C * sa;
+    A1 = dt * sa;
+    kap = dt * sa / C;
+    a0 = 1.0f + dt * C * ss;
+    a1 = dt * ss;
+    bt0 = -a1 * v2 * invC;
+    bt1 = 2.0f * a1;
+    bt2 = -a1 * invC;
+    rd0 = VEL ? 0.0f : fast_rcp(A0);
+    ra0 = VEL ? 0.0f : fast_rcp(a0);
+  }
+};
+
+// The angle sums of Steps 4 and 5, over the normalised weights (see
+// process_tile_q's source loop).
+struct CellSums {
+  float T0, T1, T2, T3, U0, U1, U2;
+  float As1, Va, Ad, Adv, AQ, Bs, Bv, Bd, Bdv, BQ;
+};
+
+// The solved cell: T^{n+1}, and the per-angle update I'' - s2 = ra (Q + rd
+// (D0 + D1 vn) + E0 + E1 vn), s2 = R + e2.
+struct CellSolve {
+  double kv, T1;
+  float D0, D1, E0, E1, e2;
+};
+
+// The per-cell solves of Steps 4 and 5.
+__device__ __forceinline__ CellSolve solve_cell(const StepArgs<float> &a, const CellIn &ci, const CellSums &s) {
+  const float C = a.C, invC = a.invC, dt = a.dt;
+  const float rho = ci.rho, sa = ci.sa, R = ci.R, v2 = ci.v2, A1 = ci.A1, kap = ci.kap, a1 = ci.a1;
+  const double T0 = ci.T0;
+  const float T0s = s.T0, T1s = s.T1, T2s = s.T2, T3s = s.T3, U0s = s.U0, U1s = s.U1, U2s = s.U2;
+  const float As1 = s.As1, Va = s.Va, Ad = s.Ad, Adv = s.Adv, AQ = s.AQ;
+  const float Bs = s.Bs, Bv = s.Bv, Bd = s.Bd, Bdv = s.Bdv, BQ = s.BQ;
+  // sum W n_i and sum W n_i n_j (normalised, from the table in double)
+  auto ms = [&](int i) { return a.msum[i][0] + a.msum[i][1]; };
+  const float *vt = ci.vt;
+  const float Vws = vt[0] * ms(1) + vt[1] * ms(2) + vt[2] * ms(3);
+  const float Gqs = vt[0] * vt[0] * ms(4) + vt[1] * vt[1] * ms(5) + vt[2] * vt[2] * ms(6) +
+                    2.0f * (vt[0] * vt[1] * ms(7) + vt[0] * vt[2] * ms(8) + vt[1] * vt[2] * ms(9));
+  const float Bw = ci.bt0 + ci.bt1 * Vws + ci.bt2 * Gqs;
+
+  // ---- Step 4 solve (sec. 4.3) in dth = theta - R ------------------------------
+  // Each row reads I'_m - theta = rd (rr - dth - kappa S + 4 A1 theta vn), so
+  // S = sum g I' (g = W (v.v + vn^2)), theta - J' and H' - S/C are affine in
+  // dth, and the energy row is kv D + c0 + c1 dth(D) = 0 in D = T - T^n with
+  // dth(D) = dth0 + ((T^n + D)^4 - (T^n)^4) / 4 pi.
+  const float Gw = v2 + Gqs;
+  const float G1 = v2 * T0s + T2s, Gr = v2 * U0s + U2s, Gv = v2 * T1s + T3s;
+  const float den = 1.0f + kap * G1, Sg = Gw + 4.0f * A1 * Gv;
+  const float S0 = (R * Sg + Gr) / den, S1 = (Sg - G1) / den;   // S = S0 + S1 dth
+  const float q1 = -4.0f * A1 * T1s;
+  const float Z0 = R * q1 + kap * S0 * T0s - U0s;               // theta - J' = Z0 + Z1 dth
+  const float Z1 = q1 + T0s + kap * S1 * T0s;
+  const float hv = Vws + 4.0f * A1 * T2s, ks = kap * T1s + invC;
+  const float Y0 = R * hv + U1s - S0 * ks;                       // H' - S/C = Y0 + Y1 dth
+  const float Y1 = hv - T1s - S1 * ks;
+  const double kv = (double)rho * a.kv_per_rho;
+  const double T0sq = T0 * T0;
+  const float dth0 = (float)(T0sq * T0sq * (1.0 / (4.0 * kPi)) - (double)R);
+  double T1 = T0;
+  float dth = dth0;
+  if (!a.hold_T) {
+    const float beta = a.P * C * (1.0f - v2 * invC * invC) * sa;
+    const float c0 = dt * (float(8.0 * kPi) * a.P * sa * Y0 + float(4.0 * kPi) * beta * Z0);
+    const float c1 = dt * (float(8.0 * kPi) * a.P * sa * Y1 + float(4.0 * kPi) * beta * Z1);
+    const float cc = c0 + c1 * dth0, c4 = c1 * float(1.0 / (4.0 * kPi));
+    // Newton on D from 0; (T^n + D)^4 - (T^n)^4 = D (4 T^3 + D (6 T^2 + D (4 T
+    // + D))) with T = T^n keeps every term of the row the size of D; the
+    // stopping tolerance is the caller's (at least 1e-6 in float), then one
+    // more step
+    const float T0f = (float)T0, kvf = (float)kv;
+    const float t2 = T0f * T0f, p3 = 4.0f * t2 * T0f, p2 = 6.0f * t2, p1 = 4.0f * T0f;
+    const float rtol = fmaxf((float)a.newton_rtol, 1e-6f);
+    const int max_it = a.newton_max_it;
+    float d = 0.0f;
+    int extra = -1, it;
+    for (it = 0; it < max_it; ++it) {
+      const float T = T0f + d;
+      const float f = fmaf(kvf, d, fmaf(c4, d * fmaf(d, fmaf(d, p1 + d, p2), p3), cc));
+      const float fp = fmaf(4.0f * c4, T * T * T, kvf);
+      float dn = d - __fdividef(f, fp);   // the next iterate corrects its last bits
+      if (!(T0f + dn > 0.0f)) dn = 0.5f * T - T0f;
+      const float step = dn - d;
+      d = dn;
+      if (extra == 0) break;
+      if (extra < 0 && fabsf(step) <= rtol * (T0f + d)) extra = 0;
+    }
+    T1 = T0 + (double)d;
+    if (!(it < max_it && T1 > 0.0)) atomicAdd(a.status, 1);
+    dth = dth0 + d * fmaf(d, fmaf(d, p1 + d, p2), p3) * float(1.0 / (4.0 * kPi));
+  }
+  const float th = R + dth;
+  const float kS = kap * (S0 + S1 * dth);
+
+  // ---- Step 5 solve (sec. 4.4) in sg = s1 + a1 C s2 and e2 = s2 - R ------------
+  // Each row reads I''_m - s2 = ra (y_m + dth - e2 - sg + 4 a1 s2 vn) with
+  // y_m = r'_m - theta = Q_m + rd (D0 + D1 vn); summing it against W (s2 =
+  // sum W I'') and against beta W (sg = sum beta W I'') gives the 2x2 system.
+  const float D0 = -(dth + kS), D1 = 4.0f * A1 * th;
+  const float Ay = AQ + D0 * Ad + D1 * Adv, By = BQ + D0 * Bd + D1 * Bdv;
+  const float fa = 4.0f * a1;
+  const float m11 = 1.0f + Bs, m12 = Bs - Bw - fa * Bv, r1 = By + dth * Bs + R * (Bw + fa * Bv);
+  const float m21 = As1, m22 = As1 - fa * Va, r2 = Ay + dth * As1 + fa * R * Va;
+  const float det = m11 * m22 - m12 * m21;
+  const float sg = (r1 * m22 - m12 * r2) / det;
+  const float e2 = (m11 * r2 - m21 * r1) / det;
+  CellSolve out;
+  out.kv = kv;
+  out.T1 = T1;
+  out.D0 = D0;
+  out.D1 = D1;
+  out.E0 = dth - e2 - sg;
+  out.E1 = fa * (R + e2);
+  out.e2 = e2;
+  return out;
+}
+
+// Writes the moments of I^{n+1} (deviation sums m against W, W n, W n n), the
+// gas sources, T^{n+1} and the next center.
+__device__ __forceinline__ void store_cell(const StepArgs<float> &a, const CellIn &ci, const CellSolve &x, long long c,
+                                           f2 mE, const f2 *mF, const f2 *mP, f2 pre0, f2 pre1, f2 pre2, float cnext) {
+  const long long N = a.N;
+  const float wn = a.wnorm, R = ci.R, invC = a.invC, rho = ci.rho;
+  const float *vin = ci.vin;
+  const double kv = x.kv, T1 = x.T1, T0 = ci.T0;
+  auto hsum = [wn](f2 x) {
+    const float t = x.x + x.y;
+    return fmaf(-t, wn, t);
+  };
+  if (a.cen_out) a.cen_out[c] = cnext;
+  a.mom_out[c] = mom_4pi_double(R, a.msum[0][0], a.msum[0][1], hsum(mE));
+  float post[3];
+  for (int i = 0; i < 3; ++i) {
+    post[i] = hsum(mF[i]);
+    a.mom_out[(1 + i) * N + c] = mom_4pi_double(R, a.msum[1 + i][0], a.msum[1 + i][1], post[i]);
+  }
+  for (int i = 0; i < 6; ++i)
+    a.mom_out[(4 + i) * N + c] = mom_4pi_double(R, a.msum[4 + i][0], a.msum[4 + i][1], hsum(mP[i]));
+
+  // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
+  const float kmom = -float(4.0 * kPi) * a.P * invC;
+  float dEK = 0.0f;
+  const float pre[3] = {hsum(pre0), hsum(pre1), hsum(pre2)};
+  for (int i = 0; i < 3; ++i) {
+    const float dmom = kmom * (post[i] - pre[i]);
+    a.dMom[i * N + c] = f2d_exact(dmom);
+    const float m0 = rho * vin[i];
+    dEK += ((m0 + dmom) * (m0 + dmom) - m0 * m0) / (2.0f * rho);
+  }
+  a.T_out[c] = T1;
+  a.dEgas[c] = kv * (T1 - T0) + (double)dEK;
+}
+
 template <bool B>
 struct BoolTag {
   static constexpr bool value = B;
@@ -223,7 +445,7 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
       return m < M ? a.inflow[face * M + m] : 0.0f;
   };
 
-  const float C = a.C, invC = a.invC, dt = a.dt;
+  const float C = a.C, invC = a.invC;
 
   // ---- shared pair table (as fill_qtable) --------------------------------------
   if constexpr (!TAB_PARAM) {
@@ -585,25 +807,16 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
 
   if (!valid) return;
 
-  // ---- per-cell constants of the implicit steps (see process_tile) -------------
-  // Steps 4 and 5 are taken in deviations from the cell's center R (the
-  // smallest I^n_m over its angles): every stored right-hand side, every
-  // angle sum and both per-cell solves carry quantities of the size of I - R
-  // rather than of I, and each per-cell solve is the exact sum of the
-  // per-angle updates that follow it.  Float rounding then scales with the
-  // spread of the intensities over angle (never above I_m itself, since R
-  // <= I_m), and the energy the T^4 solve hands to the gas is the energy
-  // the per-angle update takes from the radiation, step after step.
-  float rho = a.rho[c], sa = a.sa[c], ss = a.ss[c], vt[3] = {0, 0, 0}, vin[3] = {0, 0, 0};
-  const double T0 = a.T_in[c];
+  // ---- implicit steps of the own cell ------------------------------------------
+  CellIn ci;
+  ci.template load<VEL>(a, c);
   // the cell's center: written by the step that produced I^n, or formed
   // here from I^n (padding angles excluded)
-  float R;
   if (a.cen_in) {
-    R = a.cen_in[c];
+    ci.R = a.cen_in[c];
   } else {
     const float4 *p = I4 + c;
-    R = p[0].x;
+    float R = p[0].x;
     for (int j = 0; j < NQ; ++j) {
       const float4 q = p[(long long)j * N];
       const int left = M - 4 * j;
@@ -612,31 +825,12 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
       if (left > 2) R = fminf(R, q.z);
       if (left > 3) R = fminf(R, q.w);
     }
+    ci.R = R;
   }
-  if (VEL) {
-    for (int d = 0; d < 3; ++d) vin[d] = a.v[d * N + c];
-    if (a.estimate_v) {
-      const float E = d2f_rn(a.mom_in[c]);
-      const float h = 0.5f * dt * (sa + ss);
-      for (int d = 0; d < 3; ++d) {
-        const float Fd = d2f_rn(a.mom_in[(1 + d) * N + c]), Pdd = d2f_rn(a.mom_in[(4 + d) * N + c]);
-        const float num = rho * vin[d] + h * (C * rho * vin[d] + a.P * Fd);
-        const float den = rho + h * (C * rho + a.P * (E + Pdd) / C);
-        vt[d] = num / den;
-      }
-    } else {
-      vt[0] = vin[0]; vt[1] = vin[1]; vt[2] = vin[2];
-    }
-  }
-  const bool to_scat = ss > sa;
-  const float v2 = vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2];
-  const float A0 = 1.0f + dt * C * sa, A1 = dt * sa, kap = dt * sa / C;
-  const float a0 = 1.0f + dt * C * ss, a1 = dt * ss;
-  // beta_m = b_m + a1 C = 2 a1 vn - a1 (v.v + vn^2) / C (b_m of sec. 4.4)
-  const float bt0 = -a1 * v2 * invC, bt1 = 2.0f * a1, bt2 = -a1 * invC;
-  const float rd0 = VEL ? 0.0f : fast_rcp(A0);
-  const float ra0 = VEL ? 0.0f : fast_rcp(a0);
-  const f2 sc = dup(to_scat ? 1.0f : 0.0f), nsc = dup(to_scat ? 0.0f : 1.0f), Rv = dup(R);
+  const float A0 = ci.A0, A1 = ci.A1, a0 = ci.a0, a1 = ci.a1, bt0 = ci.bt0, bt1 = ci.bt1, bt2 = ci.bt2;
+  const float rd0 = ci.rd0, ra0 = ci.ra0;
+  const float *vt = ci.vt;
+  const f2 sc = dup(ci.to_scat ? 1.0f : 0.0f), nsc = dup(ci.to_scat ? 0.0f : 1.0f), Rv = dup(ci.R);
 
   // ---- source loop: Q_m over Delta F, every angle sum of Steps 4 and 5 ---------
   // Per angle: d = A0 - A1 vn, a' = a0 - a1 vn (rd = 1/d, ra = 1/a'), rr = r_m
@@ -733,83 +927,12 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
     const float t = x.x + x.y;
     return fmaf(-t, wn, t);
   };
-  const float T0s = hsum(T0p), T1s = hsum(T1p), T2s = hsum(T2p), T3s = hsum(T3p);
-  const float U0s = hsum(U0), U1s = hsum(U1), U2s = hsum(U2);
-  // sum W n_i and sum W n_i n_j (normalised, from the table in double)
-  auto ms = [&](int i) { return a.msum[i][0] + a.msum[i][1]; };
-  const float Vws = vt[0] * ms(1) + vt[1] * ms(2) + vt[2] * ms(3);
-  const float Gqs = vt[0] * vt[0] * ms(4) + vt[1] * vt[1] * ms(5) + vt[2] * vt[2] * ms(6) +
-                    2.0f * (vt[0] * vt[1] * ms(7) + vt[0] * vt[2] * ms(8) + vt[1] * vt[2] * ms(9));
-  const float As1 = hsum(As1k), Va = hsum(Vak), Ad = hsum(Adk), Adv = hsum(Advk), AQ = hsum(AQk);
-  const float Bs = hsum(Bsk), Bv = hsum(Bvk), Bd = hsum(Bdk), Bdv = hsum(Bdvk), BQ = hsum(BQk);
-  const float Bw = bt0 + bt1 * Vws + bt2 * Gqs;
-
-  // ---- Step 4 solve (sec. 4.3) in dth = theta - R ------------------------------
-  // Each row reads I'_m - theta = rd (rr - dth - kappa S + 4 A1 theta vn), so
-  // S = sum g I' (g = W (v.v + vn^2)), theta - J' and H' - S/C are affine in
-  // dth, and the energy row is kv D + c0 + c1 dth(D) = 0 in D = T - T^n with
-  // dth(D) = dth0 + ((T^n + D)^4 - (T^n)^4) / 4 pi.
-  const float Gw = v2 + Gqs;
-  const float G1 = v2 * T0s + T2s, Gr = v2 * U0s + U2s, Gv = v2 * T1s + T3s;
-  const float den = 1.0f + kap * G1, Sg = Gw + 4.0f * A1 * Gv;
-  const float S0 = (R * Sg + Gr) / den, S1 = (Sg - G1) / den;   // S = S0 + S1 dth
-  const float q1 = -4.0f * A1 * T1s;
-  const float Z0 = R * q1 + kap * S0 * T0s - U0s;               // theta - J' = Z0 + Z1 dth
-  const float Z1 = q1 + T0s + kap * S1 * T0s;
-  const float hv = Vws + 4.0f * A1 * T2s, ks = kap * T1s + invC;
-  const float Y0 = R * hv + U1s - S0 * ks;                       // H' - S/C = Y0 + Y1 dth
-  const float Y1 = hv - T1s - S1 * ks;
-  const double kv = (double)rho * a.kv_per_rho;
-  const double T0sq = T0 * T0;
-  const float dth0 = (float)(T0sq * T0sq * (1.0 / (4.0 * kPi)) - (double)R);
-  double T1 = T0;
-  float dth = dth0;
-  if (!a.hold_T) {
-    const float beta = a.P * C * (1.0f - v2 * invC * invC) * sa;
-    const float c0 = dt * (float(8.0 * kPi) * a.P * sa * Y0 + float(4.0 * kPi) * beta * Z0);
-    const float c1 = dt * (float(8.0 * kPi) * a.P * sa * Y1 + float(4.0 * kPi) * beta * Z1);
-    const float cc = c0 + c1 * dth0, c4 = c1 * float(1.0 / (4.0 * kPi));
-    // Newton on D from 0; (T^n + D)^4 - (T^n)^4 = D (4 T^3 + D (6 T^2 + D (4 T
-    // + D))) with T = T^n keeps every term of the row the size of D; the
-    // stopping tolerance is the caller's (at least 1e-6 in float), then one
-    // more step
-    const float T0f = (float)T0, kvf = (float)kv;
-    const float t2 = T0f * T0f, p3 = 4.0f * t2 * T0f, p2 = 6.0f * t2, p1 = 4.0f * T0f;
-    const float rtol = fmaxf((float)a.newton_rtol, 1e-6f);
-    const int max_it = a.newton_max_it;
-    float d = 0.0f;
-    int extra = -1, it;
-    for (it = 0; it < max_it; ++it) {
-      const float T = T0f + d;
-      const float f = fmaf(kvf, d, fmaf(c4, d * fmaf(d, fmaf(d, p1 + d, p2), p3), cc));
-      const float fp = fmaf(4.0f * c4, T * T * T, kvf);
-      float dn = d - f / fp;
-      if (!(T0f + dn > 0.0f)) dn = 0.5f * T - T0f;
-      const float step = dn - d;
-      d = dn;
-      if (extra == 0) break;
-      if (extra < 0 && fabsf(step) <= rtol * (T0f + d)) extra = 0;
-    }
-    T1 = T0 + (double)d;
-    if (!(it < max_it && T1 > 0.0)) atomicAdd(a.status, 1);
-    dth = dth0 + d * fmaf(d, fmaf(d, p1 + d, p2), p3) * float(1.0 / (4.0 * kPi));
-  }
-  const float th = R + dth;
-  const float kS = kap * (S0 + S1 * dth);
-
-  // ---- Step 5 solve (sec. 4.4) in sg = s1 + a1 C s2 and e2 = s2 - R ------------
-  // Each row reads I''_m - s2 = ra (y_m + dth - e2 - sg + 4 a1 s2 vn) with
-  // y_m = r'_m - theta = Q_m + rd (D0 + D1 vn); summing it against W (s2 =
-  // sum W I'') and against beta W (sg = sum beta W I'') gives the 2x2 system.
-  const float D0 = -(dth + kS), D1 = 4.0f * A1 * th;
-  const float Ay = AQ + D0 * Ad + D1 * Adv, By = BQ + D0 * Bd + D1 * Bdv;
-  const float fa = 4.0f * a1;
-  const float m11 = 1.0f + Bs, m12 = Bs - Bw - fa * Bv, r1 = By + dth * Bs + R * (Bw + fa * Bv);
-  const float m21 = As1, m22 = As1 - fa * Va, r2 = Ay + dth * As1 + fa * R * Va;
-  const float det = m11 * m22 - m12 * m21;
-  const float sg = (r1 * m22 - m12 * r2) / det;
-  const float e2 = (m11 * r2 - m21 * r1) / det;
-  const float E0c = dth - e2 - sg, E1c = fa * (R + e2);
+  CellSums s;
+  s.T0 = hsum(T0p); s.T1 = hsum(T1p); s.T2 = hsum(T2p); s.T3 = hsum(T3p);
+  s.U0 = hsum(U0); s.U1 = hsum(U1); s.U2 = hsum(U2);
+  s.As1 = hsum(As1k); s.Va = hsum(Vak); s.Ad = hsum(Adk); s.Adv = hsum(Advk); s.AQ = hsum(AQk);
+  s.Bs = hsum(Bsk); s.Bv = hsum(Bvk); s.Bd = hsum(Bdk); s.Bdv = hsum(Bdvk); s.BQ = hsum(BQk);
+  const CellSolve x = solve_cell(a, ci, s);
 
   // ---- I^{n+1} over Q_m, quadrature (sec. 3) ---------------------------------
   // The moments are sums of the stored deviations I^{n+1} - R against W, W n
@@ -838,9 +961,9 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
           rd = p_rcp(p_fma(dup(-A1), vn, dup(A0)));
           ra = p_rcp(p_fma(dup(-a1), vn, dup(a0)));
         }
-        const f2 y = p_fma(rd, VEL ? p_fma(dup(D1), vn, dup(D0)) : dup(D0), Q);     // r'_m - theta
-        const f2 z = p_add(y, VEL ? p_fma(dup(E1c), vn, dup(E0c)) : dup(E0c));
-        f2 I1 = p_add(Rv, p_fma(ra, z, dup(e2)));                                  // R + (I'' - R)
+        const f2 y = p_fma(rd, VEL ? p_fma(dup(x.D1), vn, dup(x.D0)) : dup(x.D0), Q);     // r'_m - theta
+        const f2 z = p_add(y, VEL ? p_fma(dup(x.E1), vn, dup(x.E0)) : dup(x.E0));
+        f2 I1 = p_add(Rv, p_fma(ra, z, dup(x.e2)));                                  // R + (I'' - R)
         if (2 * k >= M) I1.x = 0.0f;          // padding angles stay zero
         else cnext = fminf(cnext, I1.x);
         if (2 * k + 1 >= M) I1.y = 0.0f;
@@ -864,28 +987,7 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
       pq += N;
     }
   }
-  if (a.cen_out) a.cen_out[c] = cnext;
-  a.mom_out[c] = mom_4pi_double(R, a.msum[0][0], a.msum[0][1], hsum(mE));
-  float post[3];
-  for (int i = 0; i < 3; ++i) {
-    post[i] = hsum(mF[i]);
-    a.mom_out[(1 + i) * N + c] = mom_4pi_double(R, a.msum[1 + i][0], a.msum[1 + i][1], post[i]);
-  }
-  for (int i = 0; i < 6; ++i)
-    a.mom_out[(4 + i) * N + c] = mom_4pi_double(R, a.msum[4 + i][0], a.msum[4 + i][1], hsum(mP[i]));
-
-  // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
-  const float kmom = -float(4.0 * kPi) * a.P * invC;
-  float dEK = 0.0f;
-  const float pre[3] = {hsum(pre0), hsum(pre1), hsum(pre2)};
-  for (int i = 0; i < 3; ++i) {
-    const float dmom = kmom * (post[i] - pre[i]);
-    a.dMom[i * N + c] = f2d_exact(dmom);
-    const float m0 = rho * vin[i];
-    dEK += ((m0 + dmom) * (m0 + dmom) - m0 * m0) / (2.0f * rho);
-  }
-  a.T_out[c] = T1;
-  a.dEgas[c] = kv * (T1 - T0) + (double)dEK;
+  store_cell(a, ci, x, c, mE, mF, mP, pre0, pre1, pre2, cnext);
 }
 
 // Resident CTAs per SM a tile shape is compiled for: 512 threads per SM
