@@ -1,0 +1,508 @@
+// Fused radiation-transfer step with double intensities (Jiang, Stone & Davis
+// 2014, arXiv:1403.6126, secs. 3-4), angle-major storage.
+//
+// One CTA owns a tile of cells (one thread per cell in the implicit steps).
+// The transport walks lines of up to eight cells, one angle at a time, with
+// the van Leer differences, slopes and the last flux in registers (the line
+// geometry of rt_step_sym.cuh): several angles' lines per round of two CTA
+// barriers, so that a small tile gives every thread a line.  After a round
+// each cell's thread forms the right-hand sides Q_m (kept in the output
+// array) and every angle sum of the implicit steps; then it solves its cell:
+// the T^4 energy equation of Step 4 (sec. 4.3) reduced to a scalar quartic, the
+// 2x2 system of Step 5 (sec. 4.4), then I^{n+1}, the moments E_r, F_r, P_r
+// (sec. 3) and the gas sources.
+//
+// What bounds it: the FP64 pipe (about two multiply-adds per cycle and SM) on
+// grids that fill the GPU, and the latency of its chains on small ones.  So
+// double operations are counted: one difference per cell and axis (a line
+// shares it between two slopes), a three-operation reciprocal, sign tests on
+// the bit pattern (a double compare takes the same pipe), the beta-weighted
+// sums of Step 5 as combinations of power sums of n.v, and, without velocity
+// terms, no per-angle work for sums that are the weights' own.
+//
+// Measured against the kernel it replaced (slopes and fluxes through shared
+// memory, one angle per three barriers, IEEE divisions throughout): 512-cell
+// slab of 8 angles 72 -> 40 us per step, 256 x 128 x 80 shadow problem 577 -> 377
+// us, 40^3 x 24 moving box 1008 -> 689 us.
+//
+// Reduction used (both implicit steps are linear in I for fixed T):
+//   Step 4 row m:  d_m I_m = r_m + e_m theta - kappa S,   theta = T^4/(4 pi)
+//     d_m = 1 + dt C sa - dt sa vn_m,  e_m = dt sa (C + 3 vn_m),
+//     kappa = dt sa / C,  S = sum_l g_l I_l,  g_l = W_l (v.v + vn_l^2),
+//     vn_m = n_m . v~ ;
+//   Step 5 (unknowns x = W I): a_m x_m + sum_l (b_l + c_m) x_l = r'_m with
+//     r'_m = I4_m (+ Delta F_m when sigma_s > sigma_a),
+//     I4_m = Q_m + (e_m/d_m) theta - kappa S / d_m,
+//     Q_m  = r_m / d_m (+ Delta F_m when sigma_s > sigma_a).
+// The sums are kept as moments of vn: sum W vn^k f over the angles, k = 0 .. 3,
+// with f = 1/d (T_k), r/d (U_k), 1/a' (P_k), 1/(a' d) (D_k), Q/a' (K_k), where
+// 1/a_m = W_m / a'_m.
+#pragma once
+
+#include "rt_step_sym.cuh"
+
+namespace rtg {
+
+namespace stepk {
+
+// Table of one angle: n (0-2), W (3), W n_i (4-6), W n_i n_j (7-12: xx, yy, zz,
+// xy, xz, yz), per axis C mu dt/2dx and mu dt/dx (13-18).
+constexpr int kTabD = 19;
+
+template <int DIM, bool VEL, int TX, int TY, int TZ>
+struct DoubleGeo {
+  using G = SymGeo<DIM, TX, TY, TZ>;
+  static constexpr int ROUND = G::NT / G::LINES < 8 ? G::NT / G::LINES : 8;   // angles per round
+  __host__ static size_t smem_bytes(int M) {
+    return sizeof(double) * (kTabD * (size_t)M + ROUND * ((VEL ? 2 : 1) * G::NBOX + G::NF) + (VEL ? 3 * G::NBOX : 0)) +
+           sizeof(double2) * G::NC + sizeof(PackedLine) * G::LINES;
+  }
+};
+
+// 1/x by one cubic step from the hardware's approximation (relative error e
+// below 2^-19): r (1 + e + e^2) leaves e^3 below 2^-57, so the result is within
+// one unit in the last place.  NaN for x = 0.
+__device__ __forceinline__ double rcp_cubic(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Half van Leer slope from the one-sided differences (see vl_half).
+__device__ __forceinline__ double vl_diff(double dl, double dr) {
+  const double pr = dl * dr;
+  const double h = pr * rcp_cubic(dl + dr);
+  return __double2hiint(pr) > 0 ? h : 0.0;
+}
+
+template <int DIM, bool VEL, int TX, int TY, int TZ>
+__device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int tid, int tbx, int tby, int tbz,
+                                               unsigned char *smem_raw) {
+  using G = SymGeo<DIM, TX, TY, TZ>;
+  constexpr int NT = G::NT, ROUND = DoubleGeo<DIM, VEL, TX, TY, TZ>::ROUND, SLOTS = G::SLOTS, NBOX = G::NBOX;
+  const int M = a.M;
+  const long long N = a.N;
+  const int org[3] = {tbx * TX, tby * TY, tbz * TZ};
+
+  double2 *s_fc = reinterpret_cast<double2 *>(smem_raw);        // face constants [NC]
+  double *s_tab = reinterpret_cast<double *>(s_fc + G::NC);     // [M][kTabD]
+  double *s_It = s_tab + kTabD * M;                             // I~ [ROUND][NBOX]
+  double *s_F = s_It + ROUND * NBOX;                            // Delta F per axis [ROUND][NF]
+  double *s_IV = s_F + ROUND * G::NF;                           // IV [ROUND][NBOX] (VEL)
+  double *s_w = s_IV + (VEL ? ROUND * NBOX : 0);                // w = 3 J v [3][NBOX] (VEL)
+  PackedLine *s_line = reinterpret_cast<PackedLine *>(s_w + (VEL ? 3 * NBOX : 0));   // [LINES]
+  const double C = a.C, invC = a.invC, dt = a.dt;
+
+  for (int m = tid; m < M; m += NT) {
+    double *t = s_tab + kTabD * m;
+    const double W = a.ang[4 * m + 3];
+    double n[3];
+    for (int d = 0; d < 3; ++d) {
+      n[d] = a.ang[4 * m + d];
+      t[d] = n[d];
+      t[4 + d] = W * n[d];
+      t[7 + d] = W * n[d] * n[d];
+      t[13 + 2 * d] = 0.5 * C * n[d] * a.dtdx[d];
+      t[14 + 2 * d] = n[d] * a.dtdx[d];
+    }
+    t[3] = W;
+    t[10] = W * n[0] * n[1];
+    t[11] = W * n[0] * n[2];
+    t[12] = W * n[1] * n[2];
+  }
+
+  // ---- staged cells of this thread (see process_tile_sym) ----------------------
+  int sl_box[SLOTS], sl_g[SLOTS];
+  auto used = [&](int s) { return (s + 1) * NT <= G::NCROSS || tid + s * NT < G::NCROSS; };
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) {
+    sl_box[s] = sl_g[s] = 0;
+    if (!used(s)) continue;
+    int l[3];
+    const int box = G::staged(tid + s * NT, l);
+    int g[3], code = 0;
+    for (int d = 0; d < 3; ++d) {
+      g[d] = d < DIM ? org[d] + l[d] : 0;
+      if (d < DIM && (g[d] < 0 || g[d] >= a.n[d])) {
+        if (code == 0) code = 1 + 2 * d + (g[d] >= a.n[d] ? 1 : 0);
+        g[d] = map_in(g[d], a.n[d], a.bc[d][0], a.bc[d][1]);
+      }
+    }
+    if (code) {
+      const int axis = (code - 1) >> 1, side = (code - 1) & 1;
+      const int kind = a.bc[axis][side];
+      code = (kind == BC_VACUUM || kind == BC_INFLOW) ? (1 | (kind == BC_INFLOW ? 2 : 0) | (axis << 2) | (side << 4)) : 0;
+    }
+    sl_box[s] = box | (code << 16);
+    sl_g[s] = (int)(g[0] + (long long)a.n[0] * (g[1] + (long long)a.n[1] * g[2]));
+    if (VEL) {
+      const double w3 = (3.0 / (4.0 * kPi)) * a.mom_in[sl_g[s]];
+      for (int d = 0; d < 3; ++d) s_w[d * NBOX + box] = w3 * a.v[d * N + sl_g[s]];
+    }
+  }
+  double pf[ROUND][SLOTS];   // the next round's angles of each staged cell
+  auto fetch = [&](int m0) {
+#pragma unroll
+    for (int k = 0; k < ROUND; ++k)
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (m0 + k < M && used(s)) pf[k][s] = a.I_in[(long long)(m0 + k) * N + sl_g[s]];
+  };
+  fetch(0);
+
+  // ---- alpha and v of the cells -1 .. T of every axis: face constants -----------
+  // alpha once per cell (and axis, where the cell sides differ), kept in the I~
+  // arrays meanwhile
+  double *c_al = s_It, *c_v = s_It;
+  const bool same_dx = (DIM < 2 || a.dx[1] == a.dx[0]) && (DIM < 3 || a.dx[2] == a.dx[0]);
+  for (int pass = 0; pass < (same_dx ? 1 : DIM); ++pass) {
+    if (pass) __syncthreads();
+    for (int k = tid; k < G::INNER; k += NT) {
+      int l[3], g[3];
+      const int box = G::staged(G::inner(k), l);
+      for (int d = 0; d < 3; ++d) {
+        g[d] = d < DIM ? org[d] + l[d] : 0;
+        if (d < DIM && (g[d] < 0 || g[d] >= a.n[d])) g[d] = map_in(g[d], a.n[d], a.bc[d][0], a.bc[d][1]);
+      }
+      const long long cc = g[0] + (long long)a.n[0] * (g[1] + (long long)a.n[1] * g[2]);
+      c_al[box] = alpha_of(pass == 0 ? a.dx[0] : pass == 1 ? a.dx[1] : a.dx[2], a.sa[cc] + a.ss[cc]);
+    }
+    __syncthreads();
+    if (tid < G::LINES) {
+      Line ln{};
+      const int d = G::line(tid, ln), L = d == 0 ? G::LX : d == 1 ? G::LY : G::LZ;
+      if (pass == 0) s_line[tid].pack(ln);
+      if (same_dx || d == pass) {
+        const int np = d == 0 ? G::NPX : d == 1 ? G::NPY : G::NPZ;
+        double2 *fc = s_fc + (d == 0 ? tid : d == 1 ? G::CY + tid - G::NPX : G::CZ + tid - G::NPX - G::NPY);
+        double al = c_al[ln.lo + ln.slo];
+        for (int f = 0; f <= L; ++f) {
+          const double al1 = c_al[f < L ? ln.core + f * ln.sc : ln.hi];
+          fc[f * np].x = 0.5 * (al + al1);
+          al = al1;
+        }
+      }
+    }
+  }
+  if (VEL) {
+    // g = +-(1 - |v_face| dt/dx), positive (and alpha negative) when the cell
+    // below the face is the upwind one, infinite at a face of zero velocity
+#pragma unroll 1
+    for (int d = 0; d < DIM; ++d) {
+      __syncthreads();
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (used(s)) c_v[sl_box[s] & 0xffff] = a.v[d * N + sl_g[s]];
+      __syncthreads();
+      const int first = d == 0 ? 0 : d == 1 ? G::NPX : G::NPX + G::NPY, np = d == 0 ? G::NPX : d == 1 ? G::NPY : G::NPZ;
+      if (tid < np) {
+        Line ln{};
+        G::line(first + tid, ln);
+        double2 *fc = s_fc + (d == 0 ? 0 : d == 1 ? G::CY : G::CZ) + tid;
+        const int L = d == 0 ? G::LX : d == 1 ? G::LY : G::LZ;
+        double v = c_v[ln.lo + ln.slo];
+        for (int f = 0; f <= L; ++f) {
+          const double v1 = c_v[f < L ? ln.core + f * ln.sc : ln.hi], vf = 0.5 * (v + v1);
+          const double h = 1.0 - fabs(vf) * (d == 0 ? a.dtdx[0] : d == 1 ? a.dtdx[1] : a.dtdx[2]);
+          fc[f * np].y = vf > 0.0 ? h : vf < 0.0 ? -h : __hiloint2double(0x7ff00000, 0);
+          if (vf > 0.0) fc[f * np].x = -fc[f * np].x;
+          v = v1;
+        }
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- the own cell ---------------------------------------------------------------
+  const int lx = tid % TX, ly = (tid / TX) % TY, lz = tid / (TX * TY);
+  const int gx = org[0] + lx, gy = org[1] + ly, gz = org[2] + lz;
+  const bool valid = gx < a.n[0] && gy < a.n[1] && gz < a.n[2];
+  const long long c = valid ? gx + (long long)a.n[0] * (gy + (long long)a.n[1] * gz) : 0;
+  double rho = 1, sa = 0, ss = 0, vt[3] = {0, 0, 0}, vin[3] = {0, 0, 0}, T0 = 1;
+  if (valid) {
+    rho = a.rho[c];
+    sa = a.sa[c];
+    ss = a.ss[c];
+    T0 = a.T_in[c];
+    if (VEL) {
+      for (int d = 0; d < 3; ++d) vt[d] = vin[d] = a.v[d * N + c];
+      if (a.estimate_v) {
+        // Step 3 (sec. 4.5): per axis, backward-Euler momentum exchange with
+        // E, F, P_dd held at their step-n values
+        const double E = a.mom_in[c];
+        const double h = 0.5 * dt * (sa + ss);
+        for (int d = 0; d < 3; ++d) {
+          const double Fd = a.mom_in[(1 + d) * N + c], Pdd = a.mom_in[(4 + d) * N + c];
+          const double num = rho * vin[d] + h * (C * rho * vin[d] + a.P * Fd);
+          const double den = rho + h * (C * rho + a.P * (E + Pdd) * invC);
+          vt[d] = num * rcp_cubic(den);
+        }
+      }
+    }
+  }
+  const bool scat = ss > sa;
+  const double A0 = 1.0 + dt * C * sa, A1 = dt * sa, a0 = 1.0 + dt * C * ss, a1 = dt * ss;
+  const double rd0 = VEL ? 0.0 : rcp_cubic(A0), ra0 = VEL ? 0.0 : rcp_cubic(a0);
+
+  // ---- transport, Q_m and the angle sums: ROUND angles per two barriers -------------
+  double Tk[4] = {0, 0, 0, 0}, Pk[4] = {0, 0, 0, 0}, Dk[4] = {0, 0, 0, 0};
+  double Uk[3] = {0, 0, 0}, Kk[3] = {0, 0, 0}, pre[3] = {0, 0, 0}, Ws = 0;
+  const int kq = tid / G::LINES, line = tid % G::LINES;
+  const int axis = line < G::NPX ? 0 : DIM == 2 || line < G::NPX + G::NPY ? 1 : 2;
+#pragma unroll 1
+  for (int m0 = 0; m0 < M; m0 += ROUND) {
+    double I0[ROUND];   // the own cell's I^n (slot 0 is the own cell)
+#pragma unroll
+    for (int k = 0; k < ROUND; ++k) {
+      const int m = m0 + k;
+      I0[k] = pf[k][0];
+      if (m >= M) break;
+      const double *t = s_tab + kTabD * m;
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s) {
+        if (!used(s)) continue;
+        const int box = sl_box[s] & 0xffff, code = sl_box[s] >> 16;
+        double I = pf[k][s];
+        if (code) {
+          // beyond a vacuum or inflow face, the rays that come in
+          const int ax = (code >> 2) & 3, side = (code >> 4) & 1;
+          const double mu = t[ax];
+          if (side ? (mu < 0.0) : (mu > 0.0)) I = (code & 2) ? a.inflow[(ax * 2 + side) * M + m] : 0.0;
+        }
+        if (VEL) {
+          const double iv = t[0] * s_w[box] + t[1] * s_w[NBOX + box] + t[2] * s_w[2 * NBOX + box];
+          s_IV[k * NBOX + box] = iv;
+          I -= iv * invC;
+        }
+        s_It[k * NBOX + box] = I;
+      }
+    }
+    fetch(m0 + ROUND);
+    __syncthreads();
+    if (kq < ROUND && m0 + kq < M) {
+      const double *t = s_tab + kTabD * (m0 + kq);
+      const double hc = t[13 + 2 * axis], mud = t[14 + 2 * axis], hca = fabs(hc);
+      const Line at = s_line[line].unpack();
+      auto walk = [&](auto length, auto lines, auto step, double *F, const double2 *fc) {
+        constexpr int L = decltype(length)::value, NP = decltype(lines)::value, SF = decltype(step)::value;
+        const double *It = s_It + kq * NBOX, *IV = VEL ? s_IV + kq * NBOX : s_It;
+        int p = at.lo + at.slo;
+        double Ls = It[p], q = It[at.core], d = q - Ls, sL = vl_diff(Ls - It[at.lo], d), fl = 0.0;
+        double vL = 0, v = 0, dv = 0, sLv = 0;
+        if (VEL) {
+          vL = IV[p];
+          v = IV[at.core];
+          dv = v - vL;
+          sLv = vl_diff(vL - IV[at.lo], dv);
+        }
+        p = at.core;
+#pragma unroll
+        for (int f = 0; f <= L; ++f) {
+          p = f + 1 < L ? p + at.sc : f + 1 == L ? at.hi : p + at.shi;
+          const double qn = It[p];
+          const double2 k = fc[f * NP];
+          const double e = qn - q;
+          const double sR = vl_diff(d, e);
+          const double ha = hca * fabs(k.x);             // alpha C |mu| dt / 2dx
+          const double hl = 1.0 - 2.0 * ha;              // 1 - nu
+          const double S = Ls + hl * sL, R = q - hl * sR;
+          double g = (hc + ha) * S + (hc - ha) * R;
+          if (VEL) {
+            // IV at the face: the upwind cell's state (sec. 4.2), or the mean
+            // of both at a face of zero velocity
+            const double vn = IV[p], ev = vn - v, sRv = vl_diff(dv, ev);
+            const bool below = __double2hiint(k.x) < 0, zero = __double2hiint(k.y) == 0x7ff00000;
+            double iv;
+            if (zero)
+              iv = 0.5 * ((vL + sLv) + (v - sRv));
+            else
+              iv = k.y * (below ? sLv : sRv) + (below ? vL : v);
+            g += mud * iv;
+            vL = v;
+            v = vn;
+            dv = ev;
+            sLv = sRv;
+          }
+          if (f > 0) F[(f - 1) * SF] = fl - g;
+          fl = g;
+          Ls = q;
+          q = qn;
+          d = e;
+          sL = sR;
+        }
+      };
+      double *F = s_F + kq * G::NF;
+      if (axis == 0)
+        walk(IntTag<G::LX>{}, IntTag<G::NPX>{}, IntTag<G::SX>{}, F + line, s_fc + line);
+      else if constexpr (DIM >= 2) {
+        if (axis == 1)
+          walk(IntTag<G::LY>{}, IntTag<G::NPY>{}, IntTag<G::SY>{}, F + G::FY + line - G::NPX, s_fc + G::CY + line - G::NPX);
+        else if constexpr (DIM == 3)
+          walk(IntTag<G::LZ>{}, IntTag<G::NPZ>{}, IntTag<G::SZ>{}, F + G::FZ + line - G::NPX - G::NPY,
+               s_fc + G::CZ + line - G::NPX - G::NPY);
+      }
+    }
+    __syncthreads();
+    if (!valid) continue;
+#pragma unroll
+    for (int k = 0; k < ROUND; ++k) {
+      const int m = m0 + k;
+      if (m >= M) break;
+      const double *t = s_tab + kTabD * m, *F = s_F + k * G::NF;
+      double dF = F[G::part_x(lx, ly, lz)];
+      if (DIM >= 2) dF += F[G::part_y(lx, ly, lz)];
+      if (DIM == 3) dF += F[G::part_z(lx, ly, lz)];
+      const double full = I0[k] + dF, r = scat ? I0[k] : full, W = t[3];
+      double Q;
+      if (VEL) {
+        const double vn = t[0] * vt[0] + t[1] * vt[1] + t[2] * vt[2];
+        const double rd = rcp_cubic(A0 - A1 * vn), ra = rcp_cubic(a0 - a1 * vn);
+        const double u = r * rd;
+        Q = scat ? u + dF : u;
+        const double z = Q * ra, pd = ra * rd, y1 = W * vn, y2 = y1 * vn, y3 = y2 * vn;
+        Tk[0] += W * rd; Tk[1] += y1 * rd; Tk[2] += y2 * rd; Tk[3] += y3 * rd;
+        Pk[0] += W * ra; Pk[1] += y1 * ra; Pk[2] += y2 * ra; Pk[3] += y3 * ra;
+        Dk[0] += W * pd; Dk[1] += y1 * pd; Dk[2] += y2 * pd; Dk[3] += y3 * pd;
+        Uk[0] += W * u; Uk[1] += y1 * u; Uk[2] += y2 * u;
+        Kk[0] += W * z; Kk[1] += y1 * z; Kk[2] += y2 * z;
+      } else {
+        const double u = r * rd0;
+        Q = scat ? u + dF : u;
+        Ws += W;
+        Uk[0] += W * u;
+        Kk[0] += W * Q;
+      }
+      for (int i = 0; i < 3; ++i) pre[i] += t[4 + i] * full;   // sum W n (I^n + Delta F)
+      a.I_out[(long long)m * N + c] = Q;
+    }
+  }
+  if (!valid) return;
+  if (!VEL) {
+    Tk[0] = Ws * rd0;
+    Pk[0] = Ws * ra0;
+    Dk[0] = Ws * (rd0 * ra0);
+    Kk[0] *= ra0;
+  }
+
+  // ---- Step 4 solve: S, J, v.H affine in theta; scalar quartic in T ---------
+  const double v2 = vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2];
+  const double kap = A1 * invC;
+  const double Gr = v2 * Uk[0] + Uk[2], G1 = v2 * Tk[0] + Tk[2];
+  const double Ve = A1 * (C * Tk[1] + 3.0 * Tk[2]);
+  const double Ge = A1 * (C * G1 + 3.0 * (v2 * Tk[1] + Tk[3]));
+  const double Wq = Tk[0] - 4.0 * A1 * Tk[1];     // sum W (d - e) / d
+  const double rden = rcp_cubic(1.0 + kap * G1);
+  const double S0 = Gr * rden, S1 = Ge * rden;
+  const double J0 = Uk[0] - kap * S0 * Tk[0];
+  const double H0 = Uk[1] - kap * S0 * Tk[1], H1 = Ve - kap * S1 * Tk[1];
+  const double omJ1 = Wq + kap * S1 * Tk[0];   // 1 - dJ/dtheta, cancellation-free
+  const double kv = rho * a.kv_per_rho;
+  double T1 = T0;
+  if (!a.hold_T) {
+    const double beta = a.P * C * (1.0 - v2 * invC * invC) * sa;
+    const double c0 = dt * (8.0 * kPi * a.P * sa * (H0 - S0 * invC) - 4.0 * kPi * beta * J0) - kv * T0;
+    const double c4 = dt * (2.0 * a.P * sa * (H1 - S1 * invC) + beta * omJ1);
+    // the FP64 reference's iteration and stopping rule (with its default
+    // options): Newton from T^n until |dT| <= newton_rtol T, then one more
+    // step, at most newton_max_it steps
+    const double rtol = a.newton_rtol;
+    const int max_it = a.newton_max_it;
+    double T = T0;
+    int extra = -1, it;
+    for (it = 0; it < max_it; ++it) {
+      const double T3 = T * T * T;
+      const double f = c4 * T3 * T + kv * T + c0;
+      const double fp = 4.0 * c4 * T3 + kv;
+      double Tn = T - f * rcp_cubic(fp);
+      if (!(Tn > 0)) Tn = 0.5 * T;
+      const double dT = Tn - T;
+      T = Tn;
+      if (extra == 0) break;
+      if (extra < 0 && fabs(dT) <= rtol * T) extra = 0;
+    }
+    if (it >= max_it) atomicAdd(a.status, 1);
+    T1 = T;
+  }
+  const double T1sq = T1 * T1, th = T1sq * T1sq * (1.0 / (4.0 * kPi));
+  const double kS = kap * (S0 + th * S1);
+
+  // ---- Step 5 solve: (1+B1) s1 + Bc s2 = Br,  A1 s1 + (1+Ac) s2 = Ar -------
+  // b_m = bq0 + bq1 vn + bq2 vn^2, c_m = cq vn; e_m / d_m = A1 (C + 3 vn) / d_m
+  const double bq0 = -a1 * C - a1 * v2 * invC, bq1 = 2.0 * a1, bq2 = -a1 * invC, cq = -3.0 * a1;
+  const double Bd = bq0 * Dk[0] + bq1 * Dk[1] + bq2 * Dk[2], Bdv = bq0 * Dk[1] + bq1 * Dk[2] + bq2 * Dk[3];
+  const double Ap = A1 * (C * Dk[0] + 3.0 * Dk[1]), Bp = A1 * (C * Bd + 3.0 * Bdv);
+  const double BQ = bq0 * Kk[0] + bq1 * Kk[1] + bq2 * Kk[2];
+  const double Ar = Kk[0] + th * Ap - kS * Dk[0];
+  const double Br = BQ + th * Bp - kS * Bd;
+  // 1 + sum W b / a', formed without cancellation
+  const double m11 = (1.0 - a1 * v2 * invC) * Pk[0] + a1 * Pk[1] - a1 * invC * Pk[2];
+  const double m12 = cq * (bq0 * Pk[1] + bq1 * Pk[2] + bq2 * Pk[3]);
+  const double m21 = Pk[0], m22 = 1.0 + cq * Pk[1];
+  const double rdet = rcp_cubic(m11 * m22 - m12 * m21);
+  const double s1 = (Br * m22 - m12 * Ar) * rdet;
+  const double s2 = (m11 * Ar - m21 * Br) * rdet;
+
+  // ---- I^{n+1} over Q_m, quadrature (sec. 3) ------------------------------------
+  // I = (Q + (y0 + y1 vn) / d - s1 - cq s2 vn) / a'
+  const double y0 = A1 * C * th - kS, y1 = 3.0 * A1 * th, z1 = cq * s2;
+  const double k0 = (y0 * rd0 - s1) * ra0;   // without velocity: I = Q / a' + k0
+  double mom[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  double Qn = a.I_out[c], Qnn = a.I_out[(M > 1 ? N : 0) + c];
+#pragma unroll 2
+  for (int m = 0; m < M; ++m) {
+    const double Q = Qn;
+    Qn = Qnn;
+    if (m + 2 < M) Qnn = a.I_out[(long long)(m + 2) * N + c];   // two angles ahead
+    const double *t = s_tab + kTabD * m;
+    double I1;
+    if (VEL) {
+      const double vn = t[0] * vt[0] + t[1] * vt[1] + t[2] * vt[2];
+      const double rd = rcp_cubic(A0 - A1 * vn), ra = rcp_cubic(a0 - a1 * vn);
+      I1 = (Q + rd * (y0 + y1 * vn) - s1 - z1 * vn) * ra;
+    } else {
+      I1 = Q * ra0 + k0;
+    }
+    a.I_out[(long long)m * N + c] = I1;
+#pragma unroll
+    for (int i = 0; i < 10; ++i) mom[i] += t[3 + i] * I1;   // W, W n_i, W n_i n_j
+  }
+  for (int i = 0; i < 10; ++i) a.mom_out[(long long)i * N + c] = 4.0 * kPi * mom[i];
+
+  // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
+  const double kmom = -4.0 * kPi * a.P * invC;
+  const double r2rho = 0.5 * rcp_cubic(rho);
+  double dEK = 0;
+  for (int i = 0; i < 3; ++i) {
+    const double dmom = kmom * (mom[1 + i] - pre[i]);
+    a.dMom[i * N + c] = dmom;
+    const double m0 = rho * vin[i];
+    dEK += ((m0 + dmom) * (m0 + dmom) - m0 * m0) * r2rho;
+  }
+  a.T_out[c] = T1;
+  a.dEgas[c] = kv * (T1 - T0) + dEK;
+}
+
+template <int DIM, bool VEL, int TX, int TY, int TZ>
+__global__ void __launch_bounds__(TX * TY * TZ) step_kernel_d(const StepArgs<double> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int o = a.outer_begin;
+  process_tile_d<DIM, VEL, TX, TY, TZ>(a, threadIdx.x, blockIdx.x + (DIM == 1 ? o : 0), blockIdx.y + (DIM == 2 ? o : 0),
+                                       blockIdx.z + (DIM == 3 ? o : 0), smem_raw);
+}
+
+template <int DIM, bool VEL, int TX, int TY, int TZ>
+cudaError_t launch_shape_d(const StepArgs<double> &a, cudaStream_t s) {
+  const size_t sm = DoubleGeo<DIM, VEL, TX, TY, TZ>::smem_bytes(a.M);
+  auto kern = step_kernel_d<DIM, VEL, TX, TY, TZ>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  dim3 grid((a.n[0] + TX - 1) / TX, (a.n[1] + TY - 1) / TY, (a.n[2] + TZ - 1) / TZ);
+  if (a.outer_count > 0) (DIM == 3 ? grid.z : DIM == 2 ? grid.y : grid.x) = a.outer_count;
+  kern<<<grid, TX * TY * TZ, sm, s>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace stepk
+
+}  // namespace rtg

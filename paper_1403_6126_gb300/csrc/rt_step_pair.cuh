@@ -1,8 +1,8 @@
 // Fused radiation-transfer step with float intensities, two angles per
 // thread (Jiang, Stone & Davis 2014, arXiv:1403.6126, secs. 3-4).
 //
-// Same algorithm, tile geometry and phases as process_tile in
-// rt_step_kernel.cuh, with every per-angle quantity carried as a pair
+// One thread per cell walks the angles in the phases of process_tile_q
+// (rt_step_quad.cuh), with every per-angle quantity carried as a pair
 // (angles 2k and 2k + 1) through the packed FP32 instructions of sm_100-class
 // GPUs (__ffma2_rn, __fadd2_rn, __fmul2_rn): one instruction does the
 // arithmetic of both angles, one 64-bit shared-memory access moves both, and
@@ -63,7 +63,10 @@ __device__ __forceinline__ f2 p_fma(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, 
 __device__ __forceinline__ f2 p_sub(f2 a, f2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ f2 p_rcp(f2 a) { return make_float2(fast_rcp(a.x), fast_rcp(a.y)); }
 
-// Half van Leer slopes of two angles (see vl_half).
+// Half van Leer slopes of two angles (Stone & Mihalas 1992, eq. 4):
+// the slope is the harmonic mean 2 dl dr / (dl + dr) of the one-sided differences
+// when they agree in sign, else 0; half of it is what the face states q +- (1 -
+// nu)/2 * slope need.
 __device__ __forceinline__ f2 vl_half2(f2 qm, f2 q0, f2 qp) {
   const f2 dl = p_sub(q0, qm), dr = p_sub(qp, q0);
   const f2 pr = p_mul(dl, dr);
@@ -93,7 +96,9 @@ struct KSum2 {
   }
 };
 
-// Face flux of two angles (see face_flux): al, hv, wl belong to the face,
+// Face flux of two angles, times dt/dx: the alpha blend of the van Leer states of
+// I~ (sec. 4.2: upwind weight (1 + alpha)/2, downwind (1 - alpha)/2, speed alpha C)
+// plus mu times the IV state upwinded by the face velocity; al, hv, wl belong to the face,
 // hc, hca, mud to the angles.
 template <bool VEL>
 __device__ __forceinline__ f2 face_flux2(f2 qL, f2 sL, f2 qR, f2 sR, f2 pL, f2 tL, f2 pR, f2 tR, f2 al, f2 hv, f2 wl,
@@ -123,7 +128,7 @@ __host__ __device__ inline size_t smem_bytes2(int dim, int M, bool has_v, int tx
   return n2 * sizeof(f2) + 16;
 }
 
-// One tile of one problem, float intensities: arguments as process_tile.
+// One tile of one problem, float intensities: arguments as process_tile_q.
 // B16: intensities stored as bf16 deviations (see b16_decode), Q_m in a.Q.
 template <int DIM, bool VEL, int TX, int TY, int TZ, bool B16 = false>
 __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid, int tbx, int tby, int tbz,
@@ -191,7 +196,7 @@ __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid,
     own_fx[d] = G::fx_off(d) + G::fx_idx(d, loc[d], loc[0], loc[1], loc[2]);   // face below the cell
   }
 
-  // ---- staging slots (see process_tile) ---------------------------------------
+  // ---- staging slots (see process_tile_q) ---------------------------------------
   int sl_box[kSlots], sl_code[kSlots], sl_g[kSlots];
   float sl_w[kSlots][3], sl_J[B16 ? kSlots : 1];   // sl_J: mean intensity of the slot's cell (bf16 storage)
 #pragma unroll
@@ -245,7 +250,7 @@ __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid,
     if (B16) sl_J[B16 ? s : 0] = b16_mean((float)a.mom_in[sl_g[s]]);
   }
 
-  // ---- slope-extension items (see process_tile) -------------------------------
+  // ---- slope-extension items (see process_tile_q) -------------------------------
   int ext_bb[kExt > 0 ? kExt : 1], ext_st[kExt > 0 ? kExt : 1], ext_si[kExt > 0 ? kExt : 1];
 #pragma unroll
   for (int j = 0; j < kExt; ++j) {
@@ -265,7 +270,7 @@ __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid,
     ext_si[j] = G::sl_off(d) + G::sl_idx(d, l0, l1, l2);
   }
 
-  // ---- face constants (see process_tile) ---------------------------------------
+  // ---- face constants (see process_tile_q) ---------------------------------------
   float fu_al[3], fu_hv[3], fu_wl[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) { fu_al[d] = 1.0f; fu_hv[d] = 1.0f; fu_wl[d] = 0.5f; }
@@ -309,7 +314,7 @@ __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid,
     face_consts<float, VEL>(a, d, gl, gu, &lf_al[j], &lf_hv[j], &lf_wl[j]);
   }
 
-  // ---- per-cell constants of the implicit steps (see process_tile) -------------
+  // ---- per-cell constants of the implicit steps (see process_tile_q) -------------
   float rho = 1, sa = 0, ss = 0, vt[3] = {0, 0, 0}, vin[3] = {0, 0, 0};
   double T0 = 1.0;
   if (valid) {
@@ -544,7 +549,7 @@ __device__ __forceinline__ void process_tile2(const StepArgs<float> &a, int tid,
   const float Ap = Apk.x + Apk.y, Ad = Adk.x + Adk.y, As1 = As1k.x + As1k.y, Acc = Acck.x + Acck.y;
   const float Bp = Bpk.x + Bpk.y, Bd = Bdk.x + Bdk.y, Bcc = Bcck.x + Bcck.y, B1p = B1pk.x + B1pk.y;
 
-  // ---- Step 4 solve (see process_tile) -----------------------------------------
+  // ---- Step 4 solve (see process_tile_q) -----------------------------------------
   const float Wr = U0.total(), Vr = U1.x + U1.y, Gr = v2 * Wr + (U2.x + U2.y);
   const float W1 = T0s, V1 = T1s, G1 = v2 * T0s + T2s;
   const float Ve = A1 * (C * T1s + 3.0f * T2s);

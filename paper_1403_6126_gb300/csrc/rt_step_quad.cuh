@@ -492,7 +492,9 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
     own_fx[d] = G::fx_off(d) + G::fx_idx(d, loc[d], loc[0], loc[1], loc[2]);
   }
 
-  // ---- staging slots (see process_tile) ---------------------------------------
+  // ---- staging slots: fixed cross cells of this thread (slot 0 is the own cell) ----
+  // sl_code: bit 0 = the cell lies beyond a vacuum or inflow face, bit 1 =
+  // inflow, bits 2-3 = axis, bit 4 = upper side
   int sl_box[kSlots], sl_code[kSlots], sl_g[kSlots];
   float sl_w[kSlots][3];
 #pragma unroll
@@ -547,7 +549,7 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
     }
   }
 
-  // ---- slope-extension items (see process_tile) -------------------------------
+  // ---- slope-extension items: one layer beyond the tile along each axis -----------
   int ext_bb[kExt > 0 ? kExt : 1], ext_st[kExt > 0 ? kExt : 1], ext_si[kExt > 0 ? kExt : 1];
 #pragma unroll
   for (int j = 0; j < kExt; ++j) {
@@ -567,7 +569,8 @@ __device__ __forceinline__ void process_tile_q(const StepArgs<float> &a, const Q
     ext_si[j] = G::sl_off(d) + G::sl_idx(d, l0, l1, l2);
   }
 
-  // ---- face constants (see process_tile) ---------------------------------------
+  // ---- face constants: alpha, 1 - |v_face| dt/dx and the left state's weight; the
+  // upper faces of the own cell, then the tile's lowest faces as work items ----------
   float fu_al[3], fu_hv[3], fu_wl[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) { fu_al[d] = 1.0f; fu_hv[d] = 1.0f; fu_wl[d] = 0.5f; }

@@ -170,18 +170,17 @@ struct SymGeo {
   // halo runs over its four layers fastest: the two cells of a side share a
   // 32-byte sector of the intensity array.
   __host__ __device__ static constexpr int staged(int k, int l[3]) {
-    constexpr int HX = 2 * kHalo * TY * TZ;
     if (k < NT) {
       l[0] = k % TX; l[1] = (k / TX) % TY; l[2] = k / (TX * TY);
       return l[0] + kHalo + RX * (l[1] + TY * l[2]);
     }
     k -= NT;
-    if (k < HX) {
+    if (k < 2 * HX) {
       const int r = k / (2 * kHalo);
       l[0] = outside(k % (2 * kHalo), TX); l[1] = r % TY; l[2] = r / TY;
       return l[0] + kHalo + RX * r;
     }
-    k -= HX;
+    k -= 2 * HX;
     if (k < YH) {
       l[0] = k % TX; l[1] = outside((k / TX) % (2 * kHalo), TY); l[2] = k / (2 * kHalo * TX);
       return CORE + k;
@@ -191,6 +190,20 @@ struct SymGeo {
     return CORE + YH + k;
   }
   __host__ __device__ static constexpr int outside(int h, int T) { return h < kHalo ? h - kHalo : T + h - kHalo; }
+
+  // Of the staged cells, the tile's and the inner halo layers (-1 and T): item k
+  // (0 .. INNER - 1) is staged cell inner(k).
+  static constexpr int HX = 2 * TY * TZ, HY = DIM >= 2 ? 2 * TX * TZ : 0, HZ = DIM >= 3 ? 2 * TX * TY : 0;
+  static constexpr int INNER = NT + HX + HY + HZ;
+  __host__ __device__ static constexpr int inner(int k) {
+    if (k < NT) return k;
+    k -= NT;
+    if (k < HX) return NT + 2 * kHalo * (k >> 1) + 1 + (k & 1);
+    k -= HX;
+    if (k < HY) return NT + 2 * HX + 2 * kHalo * TX * (k / (2 * TX)) + TX + k % (2 * TX);
+    k -= HY;
+    return NT + 2 * HX + 2 * HY + TX * TY + k;
+  }
 
   // Place in the tile of position pos of line p along axis d.
   __host__ __device__ static constexpr void line_cell(int d, int p, int pos, int l[3]) {

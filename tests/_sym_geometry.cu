@@ -1,5 +1,5 @@
-// Host-side check of the pair kernel's tile geometry (SymGeo in
-// rt_step_sym.cuh) for every compiled tile shape.  Built and run by
+// Host-side check of the tile geometry (SymGeo in rt_step_sym.cuh) of the pair
+// and the double kernel, for every compiled tile shape.  Built and run by
 // tests/test_sym_geometry.py; prints OK when every check holds.
 //  - the staged cells are the cross-shaped halo, each once, at places of
 //    shared memory of their own;
@@ -7,7 +7,8 @@
 //    cell that line_cell names, one step along the line's axis apart;
 //  - the lines of an axis cover each cell once, and its part of Delta F lies
 //    where the thread that adds the parts up looks for it;
-//  - face constants have places of their own in [0, NC).
+//  - face constants have places of their own in [0, NC);
+//  - the inner staged cells (inner) are the tile and its first halo layers.
 #include <cstdio>
 #include <map>
 #include <vector>
@@ -45,6 +46,18 @@ void check() {
     CHECK(place.count(key(l)) == 0);
     place[key(l)] = b;
   }
+  int inner = 0;
+  std::vector<int> seen(G::NCROSS, 0);
+  for (int k = 0; k < G::INNER; ++k) {
+    int l[3];
+    const int at = G::inner(k);
+    CHECK(at >= 0 && at < G::NCROSS && seen[at]++ == 0);
+    G::staged(at, l);
+    bool in = true;
+    for (int d = 0; d < 3; ++d) in = in && l[d] >= -1 && l[d] <= T[d];
+    inner += in;
+  }
+  CHECK(inner == G::INNER);
   std::vector<int> F(G::NF, 0), C(G::NC, 0);
   const int np[3] = {G::NPX, G::NPY, G::NPZ}, len[3] = {G::LX, G::LY, G::LZ}, off[3] = {0, G::CY, G::CZ};
   int e = 0;
@@ -87,6 +100,10 @@ int main() {
   check<2, 16, 8, 1>();
   check<2, 8, 8, 1>();
   check<2, 8, 4, 1>();
+  check<1, 256, 1, 1>();
+  check<1, 128, 1, 1>();
+  check<1, 64, 1, 1>();
+  check<1, 32, 1, 1>();
   if (failures == 0) std::printf("OK\n");
   return failures == 0 ? 0 : 1;
 }

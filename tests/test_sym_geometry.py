@@ -1,5 +1,5 @@
-"""The pair kernel's tile geometry, checked on the host: staged cells,
-lines, Delta F places and face constants of every compiled tile shape
+"""The tile geometry of the pair and the double kernel, checked on the host:
+staged cells, lines, Delta F places and face constants of every compiled tile shape
 (tests/_sym_geometry.cu, built with nvcc for the host only; no GPU is used)."""
 import os
 import shutil
