@@ -452,9 +452,15 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
     c->host_angf[4 * i + 3] = (float)ang->w[c->order[i]];
   }
   c->host_inflowf.assign(6 * (size_t)M, 0.0f);
-  bool ok = c->fp64 ? rtg::choose_tile<double>(c->dim, M, true, &c->tile)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    delete c;
+    return fail(RT_E_CUDA, "rt_create: cannot query the device");
+  }
+  bool ok = c->fp64 ? rtg::choose_tile<double>(c->dim, M, true, c->n, c->sms, &c->tile)
             : c->bf16 ? rtg::choose_tile_b16(c->dim, M, &c->tile)
-                      : rtg::choose_tile<float>(c->dim, M, true, &c->tile);
+                      : rtg::choose_tile<float>(c->dim, M, true, c->n, c->sms, &c->tile);
   if (!ok) {
     delete c;
     return fail(RT_E_INVALID, "rt_create: too many angles for one CTA's shared memory");
@@ -637,9 +643,9 @@ rt_status rt_set_tile(rt_ctx *c, int tx, int ty, int tz) {
   if (!c) return fail(RT_E_INVALID, "rt_set_tile: NULL context");
   rtg::TileShape t{tx, ty, tz};
   if (tx == 0 && ty == 0 && tz == 0) {
-    bool ok = c->fp64 ? rtg::choose_tile<double>(c->dim, c->M, true, &t)
+    bool ok = c->fp64 ? rtg::choose_tile<double>(c->dim, c->M, true, c->n, c->sms, &t)
               : c->bf16 ? rtg::choose_tile_b16(c->dim, c->M, &t)
-                        : rtg::choose_tile<float>(c->dim, c->M, true, &t);
+                        : rtg::choose_tile<float>(c->dim, c->M, true, c->n, c->sms, &t);
     if (!ok) return fail(RT_E_INVALID, "rt_set_tile: no default tile fits");
   } else {
     bool ok;
@@ -1001,7 +1007,12 @@ rt_status rt_step_coupled(rt_ctx *c, double dt, const double *rho, const double 
   // a "plane" is the set of cells with one coordinate along it
   const int d_out = std::max(0, c->dim - 1);
   const int nz = c->n[d_out];
-  const int TZ = std::max(1, d_out == 2 ? c->tile.tz : d_out == 1 ? c->tile.ty : c->tile.tx);
+  // A layer is one tile, or in 1-D and 2-D as many as span 256 (float 512)
+  // and 16 cells: small tiles run side by side in one launch, and slabs of
+  // fewer would run them one after another.
+  const int tile_z = std::max(1, d_out == 2 ? c->tile.tz : d_out == 1 ? c->tile.ty : c->tile.tx);
+  const int per = std::max(1, (d_out == 2 ? 1 : d_out == 1 ? 16 : c->fp64 ? 256 : 512) / tile_z);
+  const int TZ = per * tile_z;
   const int layers = (nz + TZ - 1) / TZ;
   if (c->opt.device_ptrs || c->bf16 || !c->material_set || !c->intensity_set || layers < 2 ||
       c->stage_len < 10 * c->N) {
@@ -1075,7 +1086,8 @@ rt_status rt_step_coupled(rt_ctx *c, double dt, const double *rho, const double 
     cudaStream_t ks = (s & 1) ? c->xs_k : c->stream;
     RT_CUDA(cudaStreamWaitEvent(ks, c->ev_in[s], 0));
     sent = std::max(sent, upto);
-    if ((st = coupled_launch(c, dt, vel, L[s], L[s + 1], ks)) != RT_OK) return st;
+    st = coupled_launch(c, dt, vel, per * L[s], std::min(per * L[s + 1], (nz + tile_z - 1) / tile_z), ks);
+    if (st != RT_OK) return st;
     const long long c0 = (long long)L[s] * TZ * Nxy, c1 = (long long)e[s] * Nxy;
     if ((st = coupled_out(c, c0, c1, c->ev_done[s], ks, dE_gas, dMom, T_new)) != RT_OK) return st;
   }

@@ -63,13 +63,14 @@ __global__ void __launch_bounds__(TX * TY * TZ, stepk::kQMinBlocks<TX * TY * TZ>
                                                                it / (ntx * nty), smem);
 }
 
-// Per device: the scratch array's device address, and per dimension the SM
-// count and resident CTAs at the shared-memory size last set.
+// Per device: the scratch array's device address, the SM count, and per kernel
+// the resident CTAs at the shared-memory size last set.
+constexpr int kNoallocKernels = 10;
 struct DeviceCache {
   void *scratch = nullptr;
   int sms = 0;
-  size_t smem[5] = {0, 0, 0, 0, 0};   // per kernel: 1-D, 2-D, 3-D; 2-D, 3-D on opposite pairs
-  int per_sm[5] = {0, 0, 0, 0, 0};
+  size_t smem[kNoallocKernels] = {};
+  int per_sm[kNoallocKernels] = {};
 };
 struct NoallocState {
   std::mutex mu;
@@ -86,7 +87,7 @@ rt_status current_device(int *dev) {
 
 // The scratch address for the current device (looked up on its first call,
 // with the device current).
-rt_status scratch_for(int dev, unsigned char **out) {
+rt_status scratch_for(int dev, unsigned char **out, int *nsm) {
   std::lock_guard<std::mutex> lock(g_state.mu);
   DeviceCache &d = g_state.dev[dev];
   if (!d.scratch) {
@@ -102,6 +103,7 @@ rt_status scratch_for(int dev, unsigned char **out) {
     d.sms = std::max(1, sms);
   }
   *out = static_cast<unsigned char *>(d.scratch);
+  *nsm = d.sms;
   return RT_OK;
 }
 
@@ -132,15 +134,34 @@ cudaError_t launch_noalloc(Kern kern, int k, const StepArgs<float> &a, const Tab
 }
 
 template <int DIM, int TX, int TY, int TZ>
-cudaError_t launch_noalloc_quad(const StepArgs<float> &a, const NoallocTable &qt, int dev, cudaStream_t s) {
-  return launch_noalloc<TX, TY, TZ>(noalloc_kernel<DIM, TX, TY, TZ>, DIM - 1, a, qt,
+cudaError_t launch_noalloc_quad(int k, const StepArgs<float> &a, const NoallocTable &qt, int dev, cudaStream_t s) {
+  return launch_noalloc<TX, TY, TZ>(noalloc_kernel<DIM, TX, TY, TZ>, k, a, qt,
                                     stepk::smem_bytes_q(DIM, a.M, true, TX, TY, TZ, true), dev, s);
 }
 
 template <int DIM, int TX, int TY, int TZ>
-cudaError_t launch_noalloc_sym(const StepArgs<float> &a, const stepk::SymTable &tab, int dev, cudaStream_t s) {
-  return launch_noalloc<TX, TY, TZ>(noalloc_kernel_sym<DIM, TX, TY, TZ>, DIM + 1, a, tab,
+cudaError_t launch_noalloc_sym(int k, const StepArgs<float> &a, const stepk::SymTable &tab, int dev, cudaStream_t s) {
+  return launch_noalloc<TX, TY, TZ>(noalloc_kernel_sym<DIM, TX, TY, TZ>, k, a, tab,
                                     stepk::smem_bytes_gather_t<DIM, true, TX, TY, TZ>(a.M), dev, s);
+}
+
+// The tile of a context on the same grid (choose_tile), among those compiled
+// here: one step of 64 x 48 x 24 angles 39 us on 32 x 16, 31 on 16 x 8 (cold caches).
+cudaError_t launch_quad(const StepArgs<float> &a, const NoallocTable &qt, TileShape t, int dev, cudaStream_t s) {
+  if (a.dim == 3) return launch_noalloc_quad<3, 8, 8, 4>(0, a, qt, dev, s);
+  if (a.dim == 2)
+    return t.tx * t.ty >= 256 ? launch_noalloc_quad<2, 16, 16, 1>(1, a, qt, dev, s)
+                              : launch_noalloc_quad<2, 16, 8, 1>(2, a, qt, dev, s);
+  return t.tx >= 512   ? launch_noalloc_quad<1, 512, 1, 1>(3, a, qt, dev, s)
+         : t.tx >= 256 ? launch_noalloc_quad<1, 256, 1, 1>(4, a, qt, dev, s)
+         : t.tx >= 128 ? launch_noalloc_quad<1, 128, 1, 1>(5, a, qt, dev, s)
+                       : launch_noalloc_quad<1, 64, 1, 1>(6, a, qt, dev, s);
+}
+
+cudaError_t launch_pairs(const StepArgs<float> &a, const stepk::SymTable &tab, TileShape t, int dev, cudaStream_t s) {
+  if (a.dim == 3) return launch_noalloc_sym<3, 8, 8, 4>(7, a, tab, dev, s);
+  return t.tx * t.ty >= 256 ? launch_noalloc_sym<2, 16, 16, 1>(8, a, tab, dev, s)
+                            : launch_noalloc_sym<2, 16, 8, 1>(9, a, tab, dev, s);
 }
 
 }  // namespace
@@ -212,7 +233,8 @@ extern "C" rt_status rt_step_noalloc(const rt_grid *g, const rt_angles *ang, dou
   rt_status st = rtg::current_device(&dev);
   if (st != RT_OK) return st;
   unsigned char *scratch = nullptr;
-  if ((st = rtg::scratch_for(dev, &scratch)) != RT_OK) return st;
+  int sms = 0;
+  if ((st = rtg::scratch_for(dev, &scratch, &sms)) != RT_OK) return st;
   int *counter = reinterpret_cast<int *>(scratch);
 
   // the angle table as the device would round it, and the inflow table, in
@@ -270,18 +292,17 @@ extern "C" rt_status rt_step_noalloc(const rt_grid *g, const rt_angles *ang, dou
   a.outer_count = 0;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), s);   // the failure word
   if (e != cudaSuccess) return set_error(RT_E_CUDA, std::string("rt_step_noalloc: clear: ") + cudaGetErrorString(e));
+  rtg::TileShape tile{512, 1, 1};   // stays when no tile of a context fits: the table is not in shared memory here
+  if (!rtg::choose_tile<float>(g->dim, M, true, a.n, sms, &tile) && g->dim == 2) tile = {16, 16, 1};
   // the tables travel by value as launch parameters
   if (sym) {
     rtg::stepk::SymTable tab;
     rtg::stepk::fill_symtable(&tab, angf, M, a.C, a.dtdx, inflowf, order);
-    e = g->dim == 2 ? rtg::launch_noalloc_sym<2, 32, 16, 1>(a, tab, dev, s)
-                    : rtg::launch_noalloc_sym<3, 8, 8, 4>(a, tab, dev, s);
+    e = rtg::launch_pairs(a, tab, tile, dev, s);
   } else {
     rtg::NoallocTable qt;   // 22 KB
     rtg::stepk::fill_qtable(&qt, angf, M, a.C, a.dtdx, inflowf);
-    e = g->dim == 1   ? rtg::launch_noalloc_quad<1, 512, 1, 1>(a, qt, dev, s)
-        : g->dim == 2 ? rtg::launch_noalloc_quad<2, 32, 16, 1>(a, qt, dev, s)
-                      : rtg::launch_noalloc_quad<3, 8, 8, 4>(a, qt, dev, s);
+    e = rtg::launch_quad(a, qt, tile, dev, s);
   }
   if (e != cudaSuccess) return set_error(RT_E_CUDA, std::string("rt_step_noalloc: launch: ") + cudaGetErrorString(e));
   if (newton_failures) {

@@ -1,6 +1,6 @@
 // Tile choice and dispatch of the fused step kernels (rt_step_sym.cuh and
 // rt_step_quad.cuh for float intensities, rt_step_pair.cuh for their bf16 storage,
-// rt_step_kernel.cuh for double): the compiled shapes are listed in
+// rt_step_double.cuh for double): the compiled shapes are listed in
 // rt_shapes.h.
 #include "rt_shapes.h"
 #include "rt_step_sym.cuh"
@@ -59,16 +59,21 @@ bool tile_ok(int dim, int M, bool has_v, TileShape t) {
 }
 
 template <typename Real>
-bool choose_tile(int dim, int M, bool has_v, TileShape *out) {
+bool choose_tile(int dim, int M, bool has_v, const int *n, int sms, TileShape *out) {
   TileShape list[16];
-  int n = shape_list<Real>(dim, list);
-  for (int i = 0; i < n; ++i) {
-    if (fits<Real>(dim, M, has_v, list[i])) {
-      *out = list[i];
-      return true;
-    }
+  const int k = shape_list<Real>(dim, list);
+  const int least = sizeof(Real) == 4 && dim == 2 ? 128 : 64;
+  bool any = false;
+  for (int i = 0; i < k; ++i) {
+    const TileShape t = list[i];
+    if (!fits<Real>(dim, M, has_v, t)) continue;
+    if (any && (dim == 3 || t.tx * t.ty < least || t.tx * t.ty > out->tx * out->ty ||
+                (long long)((n[0] + t.tx - 1) / t.tx) * ((n[1] + t.ty - 1) / t.ty) > sms))
+      continue;
+    *out = t;
+    any = true;
   }
-  return false;
+  return any;
 }
 
 bool choose_tile_b16(int dim, int M, TileShape *out) {
@@ -127,8 +132,8 @@ cudaError_t launch_step<double>(const StepArgs<double> &a, int dim, bool has_v, 
   return launch_d(a, dim, has_v, t, s);
 }
 
-template bool choose_tile<float>(int, int, bool, TileShape *);
-template bool choose_tile<double>(int, int, bool, TileShape *);
+template bool choose_tile<float>(int, int, bool, const int *, int, TileShape *);
+template bool choose_tile<double>(int, int, bool, const int *, int, TileShape *);
 template bool tile_ok<float>(int, int, bool, TileShape);
 template int tile_candidates<float>(int, int, bool, TileShape *);
 template int tile_candidates<double>(int, int, bool, TileShape *);
