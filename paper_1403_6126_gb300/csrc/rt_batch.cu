@@ -9,8 +9,9 @@
 // angle count, so the long tiles start first and the interleave gives every
 // CTA a like share.  Steps are captured in a CUDA graph (one kernel per step)
 // and replayed.  Three tile sets are
-// compiled (rt_batch_k*.cu); rt_batch_autotune times them on the batch's own
-// members and keeps the fastest.
+// compiled (rt_batch_k*.cu); the one of 256 threads is the default, and
+// rt_batch_autotune times them on the batch's own members and keeps the
+// fastest.
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -34,7 +35,7 @@ static size_t variant_smem(const BatchVariant &v, int dim, int M, bool vel) {
 }
 
 bool batch_fits(int dim, int M, bool vel) {
-  // the default variant's tile must hold the angle set
+  // the largest variant's tile must hold the angle set
   return variant_smem(batch_variant(0), dim, M, vel) <= 227 * 1024;
 }
 
@@ -45,7 +46,7 @@ struct rt_batch {
   std::vector<rt_ctx *> ctxs;
   bool dirty = true;
   bool vel = false;
-  int nitems = 0, grid = 0, phase = 0, variant = 0;
+  int nitems = 0, grid = 0, phase = 0, variant = rtg::kBatchDefault;
   size_t smem = 0;
   rtg::WorkItem *d_items = nullptr;
   rtg::StepArgs<float> *d_desc[2] = {nullptr, nullptr};

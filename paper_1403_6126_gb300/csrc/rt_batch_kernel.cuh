@@ -23,7 +23,12 @@ struct BatchVariant {
 };
 
 constexpr int kBatchVariants = 3;
-// Variants in order: 512, 256 and 128 threads per CTA.
+// Variants in order: 512, 256 and 128 threads per CTA.  Two CTAs of 256 per SM
+// hide each other's barriers, which one of 512 cannot, and their halo is
+// smaller than four of 128 would stage: us per step 857 / 708 / 804 for 512
+// uneven slabs and squares, 102 / 88 / 89 for 64 of them, 218 / 188 / 354 for
+// squares of 64 to 192 beside cubes of 32 to 64.
+constexpr int kBatchDefault = 1;
 const BatchVariant &batch_variant(int i);
 
 template <bool VEL, int NT, int X2, int Y2, int X3, int Y3, int Z3>
