@@ -133,6 +133,7 @@ rtg::StepArgs<Real> rtg::make_args(rt_ctx *c, double dt) {
   a.rho = (const Real *)c->rho;
   a.sa = (const Real *)c->sa;
   a.ss = (const Real *)c->ss;
+  for (int d = 0; d < 3; ++d) a.alpha[d] = (const Real *)c->alpha[d];
   a.v = (const Real *)c->v;
   a.T_in = c->T;
   a.T_out = c->T;
@@ -148,10 +149,16 @@ rtg::StepArgs<Real> rtg::make_args(rt_ctx *c, double dt) {
   return a;
 }
 
+// Staging and alpha arrays: with one array per axis, up to 10 N doubles in all.
+static size_t stage_bytes(long long N, int M, size_t rs, int sides) {
+  const size_t used = sizeof(double) * (size_t)std::max<long long>(7 * N, (long long)6 * M) + rs * (size_t)N * sides;
+  return std::max(used, sizeof(double) * (size_t)std::max<long long>(10 * N, (long long)8 * M));
+}
+
 size_t rtg::context_bytes(long long N, int M, bool fp64) {
   const size_t rs = fp64 ? 8 : 4, Nz = (size_t)N, Mz = (size_t)M;
   const size_t Ms = fp64 ? Mz : 4 * (size_t)((M + 3) / 4);   // stored angles (float: quad padding)
-  const size_t stage = sizeof(double) * std::max<size_t>(10 * Nz, 8 * Mz);
+  const size_t stage = stage_bytes(N, M, rs, 3);
   const size_t centers = fp64 ? 0 : 2 * sizeof(float) * Nz;   // the float step's cell centers
   return rs * (2 * Ms * Nz + 6 * Nz + 10 * Mz) + 8 * (2 * 10 * Nz + 3 * Nz) + 16 * Nz + 2 * sizeof(int) + stage + centers;
 }
@@ -199,15 +206,27 @@ rt_status convert_in(rt_ctx *c, const double *src, void *dst, long long n) {
   return e == cudaSuccess ? RT_OK : cuda_fail(e, "convert");
 }
 
+template <typename Real>
+rtg::CellAlpha<Real> alpha_out(const rt_ctx *c) {
+  rtg::CellAlpha<Real> al{};
+  for (int d = 0; d < c->dim; ++d) {
+    bool first = true;
+    for (int k = 0; k < d; ++k) first = first && c->alpha[k] != c->alpha[d];
+    al.out[d] = first ? (Real *)c->alpha[d] : nullptr;
+    al.dx[d] = (Real)c->dx[d];
+  }
+  return al;
+}
+
 // Scan (and with convert, conversion into the context's arrays) of the gas
 // fields staged in c->stage, cells [c0, c1); flag bits go to c->flags[1].
 rt_status fields_in(rt_ctx *c, long long c0, long long c1, bool convert, cudaStream_t s) {
   cudaError_t e = c->fp64 ? rtg::launch_fields_in<double>(c->stage, c->N, c0, c1 - c0, convert, (double *)c->rho,
                                                           (double *)c->sa, (double *)c->ss, (double *)c->v, c->T,
-                                                          c->flags + 1, s)
+                                                          alpha_out<double>(c), c->flags + 1, s)
                           : rtg::launch_fields_in<float>(c->stage, c->N, c0, c1 - c0, convert, (float *)c->rho,
                                                          (float *)c->sa, (float *)c->ss, (float *)c->v, c->T,
-                                                         c->flags + 1, s);
+                                                         alpha_out<float>(c), c->flags + 1, s);
   return e == cudaSuccess ? RT_OK : cuda_fail(e, "fields");
 }
 
@@ -466,7 +485,16 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
     return fail(RT_E_INVALID, "rt_create: too many angles for one CTA's shared memory");
   }
   size_t rs = c->rs;
-  c->stage_len = std::max<long long>(10 * N, (long long)8 * M);
+  // Staging: the gas fields (7 N doubles), the inflow table (6 M).  Behind it,
+  // alpha of each cell for every distinct cell side, in step precision.
+  c->stage_len = std::max<long long>(7 * N, (long long)6 * M);
+  int sides = 0, side_of[3] = {0, 0, 0};
+  for (int d = 0; d < 3; ++d) {
+    side_of[d] = sides;
+    for (int k = d - 1; k >= 0; --k)
+      if ((float)c->dx[k] == (float)c->dx[d] && (!c->fp64 || c->dx[k] == c->dx[d])) side_of[d] = side_of[k];
+    if (d < c->dim && side_of[d] == sides) ++sides;
+  }
   const size_t Nz = (size_t)N, Mz = (size_t)M;
   struct {
     void **p;
@@ -477,7 +505,7 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
       {&c->ss, rs * Nz},         {&c->v, rs * 3 * Nz},             {(void **)&c->T, 8 * Nz},
       {(void **)&c->dEgas, 8 * Nz}, {(void **)&c->dMom, 8 * 3 * Nz}, {&c->ang, rs * 4 * Mz},
       {&c->inflow, rs * 6 * Mz}, {(void **)&c->flags, 2 * sizeof(int)},
-      {(void **)&c->stage, sizeof(double) * (size_t)c->stage_len},
+      {(void **)&c->stage, stage_bytes(N, M, rs, sides)},
       {(void **)&c->qscr, c->bf16 ? sizeof(float) * Mz * Nz : 0},
       {(void **)&c->cen[0], c->quad ? sizeof(float) * Nz : 0},
       {(void **)&c->cen[1], c->quad ? sizeof(float) * Nz : 0},
@@ -491,6 +519,8 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
       return fail(RT_E_NOMEM, "rt_create: device allocation failed");
     }
   }
+  if (c->fp64 || (c->sym && c->dim == 3))   // the kernels that read it
+    for (int d = 0; d < c->dim; ++d) c->alpha[d] = (char *)(c->stage + c->stage_len) + rs * Nz * side_of[d];
   // angle table [M][4] = (n_x, n_y, n_z, W) and zero inflow, via the stage
   std::vector<double> tab(4 * (size_t)M);
   for (int i = 0; i < M; ++i) {
@@ -862,6 +892,9 @@ rt_status rt_load_state(rt_ctx *c, const void *buf, size_t bytes) {
   // parameters), the batch kernel from the device table
   if (rt_status st = inflow_tables(c); st != RT_OK) return st;
   RT_CUDA(cudaMemsetAsync(c->flags, 0, 2 * sizeof(int), c->stream));
+  if (c->alpha[0])
+    RT_CUDA(c->fp64 ? rtg::launch_alpha<double>((const double *)c->sa, (const double *)c->ss, c->N, alpha_out<double>(c), c->stream)
+                    : rtg::launch_alpha<float>((const float *)c->sa, (const float *)c->ss, c->N, alpha_out<float>(c), c->stream));
   // the float step's cell centers are a function of the intensity: formed
   // again rather than saved
   if (c->quad) RT_CUDA(rtg::launch_centers((const float *)c->I[c->cur], c->M, c->N, c->cen[c->cur], c->stream));
@@ -1015,7 +1048,7 @@ rt_status rt_step_coupled(rt_ctx *c, double dt, const double *rho, const double 
   const int TZ = per * tile_z;
   const int layers = (nz + TZ - 1) / TZ;
   if (c->opt.device_ptrs || c->bf16 || !c->material_set || !c->intensity_set || layers < 2 ||
-      c->stage_len < 10 * c->N) {
+      c->stage_len < 7 * c->N) {
     // the three calls in turn
     rt_status st = rt_set_material(c, rho, T, v, sa, ss);
     if (st == RT_E_NONFINITE) c->material_set = false;

@@ -4,27 +4,13 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
-#include "rt_internal.h"
+#include "rt_aux.cuh"
 
 namespace rtg {
 
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
-
-int grid_for(long long n, int threads) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
-  }
-  long long want = (n + threads - 1) / threads;
-  long long cap = (long long)sms * 8;
-  if (want < 1) want = 1;
-  return (int)(want < cap ? want : cap);
-}
 
 template <typename Real>
 __global__ void convert_in_kernel(const double *__restrict__ src, Real *__restrict__ dst, long long n) {
@@ -211,17 +197,6 @@ __global__ void eddington_kernel(const double *__restrict__ mom, double *__restr
   }
 }
 
-// Range tests on the IEEE-754 bit pattern u of a double, in integer
-// arithmetic (FP64 compares run at GB300's low FP64 rate): the finite
-// values are the patterns with |u| below that of +infinity; the positive
-// ones are 0 < u below +infinity; the non-negative ones add -0.
-constexpr unsigned long long kInfBits = 0x7FF0000000000000ull, kAbsMask = 0x7FFFFFFFFFFFFFFFull,
-                             kNegZero = 0x8000000000000000ull;
-__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
-__device__ __forceinline__ bool finite_bits(unsigned long long u) { return (u & kAbsMask) < kInfBits; }
-__device__ __forceinline__ bool positive_bits(unsigned long long u) { return u - 1ull < kInfBits - 1ull; }
-__device__ __forceinline__ bool nonneg_bits(unsigned long long u) { return u < kInfBits || u == kNegZero; }
-
 __global__ void check_kernel(const double *__restrict__ x, long long n, double lo, int strict, int nzbit, int *flag) {
   int bits = 0;
   const bool zero_lo = lo == 0.0;
@@ -239,57 +214,7 @@ __global__ void check_kernel(const double *__restrict__ x, long long n, double l
   if (threadIdx.x == 0 && (bad || nonzero)) atomicOr(flag, (bad ? 1 : 0) | (nonzero ? nzbit : 0));
 }
 
-// Gas fields staged as doubles (stage: rho, T, v_x, v_y, v_z, sigma_a,
-// sigma_s, N each), cells [c0, c0 + n): bit 0 of *flag for a value out of
-// range (rho, T > 0; sigma >= 0; all finite), bit 1 for a nonzero velocity;
-// with CONVERT also the context's arrays (Real, T in double).
-template <typename Real, bool CONVERT>
-__global__ void fields_in_kernel(const double *__restrict__ stage, long long N, long long c0, long long n,
-                                 Real *__restrict__ rho, Real *__restrict__ sa, Real *__restrict__ ss,
-                                 Real *__restrict__ v, double *__restrict__ T, int *flag) {
-  int bits = 0;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-    const long long i = c0 + k;
-    const double r = stage[i], t = stage[N + i], vx = stage[2 * N + i], vy = stage[3 * N + i],
-                 vz = stage[4 * N + i], a = stage[5 * N + i], s = stage[6 * N + i];
-    const unsigned long long ux = bits_of(vx), uy = bits_of(vy), uz = bits_of(vz);
-    if (!(positive_bits(bits_of(r)) && positive_bits(bits_of(t)) && nonneg_bits(bits_of(a)) &&
-          nonneg_bits(bits_of(s)) && finite_bits(ux) && finite_bits(uy) && finite_bits(uz)))
-      bits |= 1;
-    if (((ux | uy | uz) & kAbsMask) != 0) bits |= 2;
-    if (CONVERT) {
-      rho[i] = (Real)r;
-      sa[i] = (Real)a;
-      ss[i] = (Real)s;
-      v[i] = (Real)vx;
-      v[N + i] = (Real)vy;
-      v[2 * N + i] = (Real)vz;
-      T[i] = t;
-    }
-  }
-  const int bad = __syncthreads_or(bits & 1), nonzero = __syncthreads_or(bits & 2);
-  if (threadIdx.x == 0 && (bad || nonzero)) atomicOr(flag, (bad ? 1 : 0) | (nonzero ? 2 : 0));
-}
-
-
 }  // namespace
-
-template <typename Real>
-cudaError_t launch_fields_in(const double *stage, long long N, long long c0, long long n, bool convert, Real *rho,
-                             Real *sa, Real *ss, Real *v, double *T, int *flag, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  if (convert)
-    fields_in_kernel<Real, true><<<grid_for(n, 256), 256, 0, s>>>(stage, N, c0, n, rho, sa, ss, v, T, flag);
-  else
-    fields_in_kernel<Real, false><<<grid_for(n, 256), 256, 0, s>>>(stage, N, c0, n, rho, sa, ss, v, T, flag);
-  return cudaGetLastError();
-}
-
-
-template cudaError_t launch_fields_in<float>(const double *, long long, long long, long long, bool, float *, float *,
-                                             float *, float *, double *, int *, cudaStream_t);
-template cudaError_t launch_fields_in<double>(const double *, long long, long long, long long, bool, double *,
-                                              double *, double *, double *, double *, int *, cudaStream_t);
 
 template <typename Real>
 cudaError_t launch_convert_in(const double *src, Real *dst, long long n, cudaStream_t s) {

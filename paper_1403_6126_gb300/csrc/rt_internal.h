@@ -38,6 +38,10 @@ struct StepArgs {
   const Real *I_in;
   Real *I_out;
   const Real *rho, *sa, *ss;  // [N]
+  // alpha of each cell for the cell side of each axis [N] (one array where the
+  // sides are equal), for the double kernel and the 3-D pair kernel of a context;
+  // the others form it from sa and ss.
+  const Real *alpha[3];
   const Real *v;      // [3][N]
   const double *T_in; // [N]
   double *T_out;      // [N]
@@ -97,6 +101,14 @@ inline void table_moment_sums(const float *ang4, int M, float out[10][2]) {
     out[k][1] = (float)(v - (double)out[k][0]);
   }
 }
+
+// Where alpha of each cell goes: one array per distinct cell side, null for
+// the others.
+template <typename Real>
+struct CellAlpha {
+  Real *out[3];
+  Real dx[3];
+};
 
 struct TileShape {
   int tx, ty, tz;
@@ -204,9 +216,14 @@ cudaError_t launch_check(const double *x, long long n, double lo, int strict, in
 // Scan of the gas fields staged as doubles (stage: rho, T, v_x, v_y, v_z,
 // sigma_a, sigma_s, N each) over cells [c0, c0 + n) into *flag (bit 0: a
 // value out of range, bit 1: some v != 0); with convert also the copy into
-// the context's arrays (rho, sigma_a, sigma_s, v in Real; T in double).
+// the context's arrays (rho, sigma_a, sigma_s, v in Real; T in double) and
+// alpha of those cells.
 template <typename Real>
 cudaError_t launch_fields_in(const double *stage, long long N, long long c0, long long n, bool convert, Real *rho,
-                             Real *sa, Real *ss, Real *v, double *T, int *flag, cudaStream_t s);
+                             Real *sa, Real *ss, Real *v, double *T, const CellAlpha<Real> &al, int *flag,
+                             cudaStream_t s);
+// alpha of N cells from their opacities.
+template <typename Real>
+cudaError_t launch_alpha(const Real *sa, const Real *ss, long long N, const CellAlpha<Real> &al, cudaStream_t s);
 
 }  // namespace rtg

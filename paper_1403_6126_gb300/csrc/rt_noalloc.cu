@@ -275,6 +275,7 @@ extern "C" rt_status rt_step_noalloc(const rt_grid *g, const rt_angles *ang, dou
   a.rho = f->rho;
   a.sa = f->sigma_a;
   a.ss = f->sigma_s;
+  for (int d = 0; d < 3; ++d) a.alpha[d] = nullptr;
   a.v = f->v;
   a.T_in = f->T;
   a.T_out = f->T;

@@ -152,7 +152,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   fetch(0);
 
   // ---- alpha and v of the cells -1 .. T of every axis: face constants -----------
-  // alpha once per cell (and axis, where the cell sides differ), kept in the I~
+  // alpha of each cell (per axis where the cell sides differ), kept in the I~
   // arrays meanwhile
   double *c_al = s_It, *c_v = s_It;
   const bool same_dx = (DIM < 2 || a.dx[1] == a.dx[0]) && (DIM < 3 || a.dx[2] == a.dx[0]);
@@ -166,7 +166,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
         if (d < DIM && (g[d] < 0 || g[d] >= a.n[d])) g[d] = map_in(g[d], a.n[d], a.bc[d][0], a.bc[d][1]);
       }
       const long long cc = g[0] + (long long)a.n[0] * (g[1] + (long long)a.n[1] * g[2]);
-      c_al[box] = alpha_of(pass == 0 ? a.dx[0] : pass == 1 ? a.dx[1] : a.dx[2], a.sa[cc] + a.ss[cc]);
+      c_al[box] = (pass == 0 ? a.alpha[0] : pass == 1 ? a.alpha[1] : a.alpha[2])[cc];
     }
     __syncthreads();
     if (tid < G::LINES) {

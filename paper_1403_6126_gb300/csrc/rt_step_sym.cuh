@@ -527,13 +527,26 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
   fetch(0, 0);
   {
     // every load before the first store to shared memory: one latency
-    float st[SLOTS], v[SLOTS][3];
+    // (in 3-D alpha comes with the context's fields: gas loop of 96 x 80 x 72 x 24
+    // angles 264 -> 257 us; in 2-D, where one CTA per SM waits for every load, forming it
+    // here is faster, 866 against 900 us for 40 steps of 128^2 x 24: sa and ss are then
+    // in L1 when the cell's own fields are read)
+    constexpr bool KEPT = DIM == 3 && !GATHER;
+    float st[SLOTS], al[SLOTS][3], v[SLOTS][3];
     double E[SLOTS];
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
       if (!used(s)) continue;
       const long long cc = sl_g[s];
-      st[s] = a.sa[cc] + a.ss[cc];
+      if constexpr (!KEPT) {
+        st[s] = a.sa[cc] + a.ss[cc];
+      } else {
+        al[s][0] = a.alpha[0][cc];
+        if (!same_dx) {
+          al[s][1] = a.alpha[1][cc];
+          if (DIM == 3) al[s][2] = a.alpha[2][cc];
+        }
+      }
       if (VEL) {
         E[s] = a.mom_in[cc];
 #pragma unroll
@@ -544,10 +557,10 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
     for (int s = 0; s < SLOTS; ++s) {
       if (!used(s)) continue;
       const int box = sl_box[s] & 0xffff;
-      c_al[box] = alpha_of(a.dx[0], st[s]);
+      c_al[box] = KEPT ? al[s][0] : alpha_of(a.dx[0], st[s]);
       if (!same_dx) {   // cells of unequal sides: one alpha per axis
-        c_al[NBOX + box] = alpha_of(a.dx[1], st[s]);
-        if (DIM == 3) c_al[2 * NBOX + box] = alpha_of(a.dx[2], st[s]);
+        c_al[NBOX + box] = KEPT ? al[s][1] : alpha_of(a.dx[1], st[s]);
+        if (DIM == 3) c_al[2 * NBOX + box] = KEPT ? al[s][2] : alpha_of(a.dx[2], st[s]);
       }
       if (VEL) {
         const float w3 = float(3.0 / (4.0 * kPi)) * d2f_rn(E[s]);
