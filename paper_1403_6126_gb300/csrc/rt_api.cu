@@ -221,19 +221,14 @@ rtg::CellAlpha<Real> alpha_out(const rt_ctx *c) {
 // Scan (and with convert, conversion into the context's arrays) of the gas
 // fields staged in c->stage, cells [c0, c1); flag bits go to c->flags[1].
 rt_status fields_in(rt_ctx *c, long long c0, long long c1, bool convert, cudaStream_t s) {
-  cudaError_t e = c->fp64 ? rtg::launch_fields_in<double>(c->stage, c->N, c0, c1 - c0, convert, (double *)c->rho,
+  const rtg::FieldSrc src{c->stage, c->stage + c->N, c->stage + 2 * c->N, c->stage + 5 * c->N, c->stage + 6 * c->N};
+  cudaError_t e = c->fp64 ? rtg::launch_fields_in<double>(src, c->N, c0, c1 - c0, convert, (double *)c->rho,
                                                           (double *)c->sa, (double *)c->ss, (double *)c->v, c->T,
                                                           alpha_out<double>(c), c->flags + 1, s)
-                          : rtg::launch_fields_in<float>(c->stage, c->N, c0, c1 - c0, convert, (float *)c->rho,
+                          : rtg::launch_fields_in<float>(src, c->N, c0, c1 - c0, convert, (float *)c->rho,
                                                          (float *)c->sa, (float *)c->ss, (float *)c->v, c->T,
                                                          alpha_out<float>(c), c->flags + 1, s);
   return e == cudaSuccess ? RT_OK : cuda_fail(e, "fields");
-}
-
-rt_status convert_out(rt_ctx *c, const void *src, double *dst, long long n) {
-  cudaError_t e = c->fp64 ? rtg::launch_convert_out<double>((const double *)src, dst, n, c->stream)
-                          : rtg::launch_convert_out<float>((const float *)src, dst, n, c->stream);
-  return e == cudaSuccess ? RT_OK : cuda_fail(e, "convert");
 }
 
 // Moments of the intensity just set (for bf16 storage: of the float field in
@@ -259,6 +254,19 @@ rt_status fetch(rt_ctx *c, const double *src, double *dst, long long n) {
     RT_CUDA(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   }
   return RT_OK;
+}
+
+// Whether a kernel may access the caller's array p (device_ptrs): doubles on an
+// 8-byte boundary in this device's own memory.  Others (another device's,
+// host memory reached through unified addressing) go by copies.
+bool in_place(const rt_ctx *c, const void *p) {
+  if (!c->opt.device_ptrs || (reinterpret_cast<uintptr_t>(p) & 7) != 0) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == c->dev;
 }
 
 // Queues the copy of n doubles from the device buffer src to the caller;
@@ -471,9 +479,8 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
     c->host_angf[4 * i + 3] = (float)ang->w[c->order[i]];
   }
   c->host_inflowf.assign(6 * (size_t)M, 0.0f);
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+  if (cudaGetDevice(&c->dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev) != cudaSuccess) {
     delete c;
     return fail(RT_E_CUDA, "rt_create: cannot query the device");
   }
@@ -551,17 +558,21 @@ rt_status rt_set_material(rt_ctx *c, const double *rho, const double *T, const d
   if (!c || !rho || !T || !v || !sa || !ss) return fail(RT_E_INVALID, "rt_set_material: NULL argument");
   const long long N = c->N;
   if (c->stage_len < 7 * N) return fail(RT_E_STATE, "rt_set_material: staging buffer too small");
-  double *s_rho = c->stage, *s_T = c->stage + N, *s_v = c->stage + 2 * N, *s_sa = c->stage + 5 * N,
-         *s_ss = c->stage + 6 * N;
   rt_status st;
-  if ((st = fetch(c, rho, s_rho, N)) != RT_OK) return st;
-  if ((st = fetch(c, T, s_T, N)) != RT_OK) return st;
-  if ((st = fetch(c, v, s_v, 3 * N)) != RT_OK) return st;
-  if ((st = fetch(c, sa, s_sa, N)) != RT_OK) return st;
-  if ((st = fetch(c, ss, s_ss, N)) != RT_OK) return st;
   // scan: bit 0 = a value out of range or non-finite, bit 1 = some v != 0
   RT_CUDA(cudaMemsetAsync(c->flags + 1, 0, sizeof(int), c->stream));
-  if ((st = fields_in(c, 0, N, false, c->stream)) != RT_OK) return st;
+  if (in_place(c, rho) && in_place(c, T) && in_place(c, v) && in_place(c, sa) && in_place(c, ss)) {
+    // one pass stages and scans device arrays that a kernel may read (gas loop of
+    // 96 x 80 x 72 cells x 24 angles 233 us, with five copies and a scan 257)
+    RT_CUDA(rtg::launch_fields_stage({rho, T, v, sa, ss}, N, c->stage, c->flags + 1, c->stream));
+  } else {
+    if ((st = fetch(c, rho, c->stage, N)) != RT_OK) return st;
+    if ((st = fetch(c, T, c->stage + N, N)) != RT_OK) return st;
+    if ((st = fetch(c, v, c->stage + 2 * N, 3 * N)) != RT_OK) return st;
+    if ((st = fetch(c, sa, c->stage + 5 * N, N)) != RT_OK) return st;
+    if ((st = fetch(c, ss, c->stage + 6 * N, N)) != RT_OK) return st;
+    if ((st = fields_in(c, 0, N, false, c->stream)) != RT_OK) return st;
+  }
   int flag = 0;
   RT_CUDA(cudaMemcpyAsync(&flag, c->flags + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   RT_CUDA(cudaStreamSynchronize(c->stream));
@@ -1157,6 +1168,13 @@ rt_status rt_get_intensity(rt_ctx *c, double *I) {
   if (!c || !I) return fail(RT_E_INVALID, "rt_get_intensity: NULL argument");
   if (!c->intensity_set) return fail(RT_E_STATE, "rt_get_intensity: no intensity yet");
   long long total = (long long)c->M * c->N, chunk = c->stage_len;
+  if (c->fp64) return deliver(c, (const double *)c->I[c->cur], I, total);
+  if (c->quad && in_place(c, I)) {
+    rtg::AngleMap order{};
+    for (int i = 0; i < c->M; ++i) order.slot[i] = (unsigned char)c->order[i];
+    RT_CUDA(rtg::launch_intensity_out((const float *)c->I[c->cur], I, c->M, c->N, order, c->stream));
+    return RT_OK;
+  }
   for (long long off = 0; off < total; off += chunk) {
     long long n = std::min(chunk, total - off);
     rt_status st = RT_OK;
@@ -1164,13 +1182,10 @@ rt_status rt_get_intensity(rt_ctx *c, double *I) {
       cudaError_t e = rtg::launch_decode_b16((const unsigned short *)c->I[c->cur], c->mom[c->cur], c->stage, off, n,
                                              c->N, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "decode");
-    } else if (c->quad) {
+    } else {
       cudaError_t e = rtg::launch_quad_out((const float *)c->I[c->cur], c->stage, off, n, c->N, c->map, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "quad layout");
-    } else {
-      st = convert_out(c, (const char *)c->I[c->cur] + off * c->rs, c->stage, n);
     }
-    if (st != RT_OK) return st;
     if ((st = deliver(c, c->stage, I + off, n)) != RT_OK) return st;
   }
   return RT_OK;

@@ -30,7 +30,7 @@ struct rt_ctx {
   float *cen[2] = {nullptr, nullptr};   // float step: each cell's smallest intensity over angles [N]
   bool has_v = false, material_set = false, intensity_set = false;
   rtg::TileShape tile{0, 0, 0};
-  int sms = 0;        // SMs of the context's device
+  int dev = 0, sms = 0;   // the context's device and its SMs
   // device state (Real = double or float)
   void *I[2] = {nullptr, nullptr};
   double *mom[2] = {nullptr, nullptr};   // E, F, P [10][N], double for every precision

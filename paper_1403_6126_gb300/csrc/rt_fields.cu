@@ -23,26 +23,37 @@ __device__ __forceinline__ void store_alpha(const CellAlpha<Real> &al, long long
     if (al.out[k]) al.out[k][i] = stepk::alpha_of(al.dx[k], st);
 }
 
-// Gas fields staged as doubles (stage: rho, T, v_x, v_y, v_z, sigma_a,
-// sigma_s, N each), cells [c0, c0 + n): bit 0 of *flag for a value out of
+// Gas fields in doubles (N each; v three times N), cells [c0, c0 + n): bit 0 of *flag for a value out of
 // range (rho, T > 0; sigma >= 0; all finite), bit 1 for a nonzero velocity;
-// with CONVERT also the context's arrays (Real, T in double) and alpha (sec. 4.1)
-// of each cell for every distinct cell side dx.
-template <typename Real, bool CONVERT>
-__global__ void fields_in_kernel(const double *__restrict__ stage, long long N, long long c0, long long n,
+// with kConvert also the context's arrays (Real, T in double) and alpha (sec. 4.1)
+// of each cell for every distinct cell side dx; with kStage also a copy of
+// the fields in stage, so that the caller's arrays are free once it is done.
+enum FieldsMode { kScan, kConvert, kStage };
+
+template <typename Real, int MODE>
+__global__ void fields_in_kernel(const FieldSrc src, long long N, long long c0, long long n,
                                  Real *__restrict__ rho, Real *__restrict__ sa, Real *__restrict__ ss,
-                                 Real *__restrict__ v, double *__restrict__ T, CellAlpha<Real> al, int *flag) {
+                                 Real *__restrict__ v, double *__restrict__ T, CellAlpha<Real> al, double *__restrict__ stage, int *flag) {
   int bits = 0;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
     const long long i = c0 + k;
-    const double r = stage[i], t = stage[N + i], vx = stage[2 * N + i], vy = stage[3 * N + i],
-                 vz = stage[4 * N + i], a = stage[5 * N + i], s = stage[6 * N + i];
+    const double r = src.rho[i], t = src.T[i], vx = src.v[i], vy = src.v[N + i], vz = src.v[2 * N + i], a = src.sa[i],
+                 s = src.ss[i];
     const unsigned long long ux = bits_of(vx), uy = bits_of(vy), uz = bits_of(vz);
     if (!(positive_bits(bits_of(r)) && positive_bits(bits_of(t)) && nonneg_bits(bits_of(a)) &&
           nonneg_bits(bits_of(s)) && finite_bits(ux) && finite_bits(uy) && finite_bits(uz)))
       bits |= 1;
     if (((ux | uy | uz) & kAbsMask) != 0) bits |= 2;
-    if (CONVERT) {
+    if (MODE == kStage) {
+      stage[i] = r;
+      stage[N + i] = t;
+      stage[2 * N + i] = vx;
+      stage[3 * N + i] = vy;
+      stage[4 * N + i] = vz;
+      stage[5 * N + i] = a;
+      stage[6 * N + i] = s;
+    }
+    if (MODE == kConvert) {
       rho[i] = (Real)r;
       sa[i] = (Real)a;
       ss[i] = (Real)s;
@@ -66,23 +77,29 @@ __global__ void alpha_kernel(const Real *__restrict__ sa, const Real *__restrict
 }  // namespace
 
 template <typename Real>
-cudaError_t launch_fields_in(const double *stage, long long N, long long c0, long long n, bool convert, Real *rho,
+cudaError_t launch_fields_in(const FieldSrc &src, long long N, long long c0, long long n, bool convert, Real *rho,
                              Real *sa, Real *ss, Real *v, double *T, const CellAlpha<Real> &al, int *flag, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (convert)
-    fields_in_kernel<Real, true><<<grid_for(n, 256), 256, 0, s>>>(stage, N, c0, n, rho, sa, ss, v, T, al, flag);
+    fields_in_kernel<Real, kConvert><<<grid_for(n, 256), 256, 0, s>>>(src, N, c0, n, rho, sa, ss, v, T, al, nullptr, flag);
   else
-    fields_in_kernel<Real, false><<<grid_for(n, 256), 256, 0, s>>>(stage, N, c0, n, rho, sa, ss, v, T, al, flag);
+    fields_in_kernel<Real, kScan><<<grid_for(n, 256), 256, 0, s>>>(src, N, c0, n, rho, sa, ss, v, T, al, nullptr, flag);
   return cudaGetLastError();
 }
 
 
-template cudaError_t launch_fields_in<float>(const double *, long long, long long, long long, bool, float *, float *,
+template cudaError_t launch_fields_in<float>(const FieldSrc &, long long, long long, long long, bool, float *, float *,
                                              float *, float *, double *, const CellAlpha<float> &, int *,
                                              cudaStream_t);
-template cudaError_t launch_fields_in<double>(const double *, long long, long long, long long, bool, double *,
+template cudaError_t launch_fields_in<double>(const FieldSrc &, long long, long long, long long, bool, double *,
                                               double *, double *, double *, double *, const CellAlpha<double> &,
                                               int *, cudaStream_t);
+
+cudaError_t launch_fields_stage(const FieldSrc &src, long long N, double *stage, int *flag, cudaStream_t s) {
+  fields_in_kernel<double, kStage>
+      <<<grid_for(N, 256), 256, 0, s>>>(src, N, 0, N, nullptr, nullptr, nullptr, nullptr, nullptr, {}, stage, flag);
+  return cudaGetLastError();
+}
 
 template <typename Real>
 cudaError_t launch_alpha(const Real *sa, const Real *ss, long long N, const CellAlpha<Real> &al, cudaStream_t s) {

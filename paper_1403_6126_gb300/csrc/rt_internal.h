@@ -176,8 +176,6 @@ struct AngleMap {
 // Elementwise helpers (all stream-ordered).
 template <typename Real>
 cudaError_t launch_convert_in(const double *src, Real *dst, long long n, cudaStream_t s);
-template <typename Real>
-cudaError_t launch_convert_out(const Real *src, double *dst, long long n, cudaStream_t s);
 // Isotropic equilibrium T^4/(4 pi): angle-major [M][N] (double), or the
 // quad-interleaved float layout with zero padding (quad = true).
 template <typename Real>
@@ -198,6 +196,10 @@ cudaError_t launch_quad_in(const double *src, float *dst, long long off, long lo
                            cudaStream_t s);
 cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, const AngleMap &map,
                             cudaStream_t s);
+// Every angle of the quad layout to the caller's [M][N] doubles (order.slot: the
+// caller's index of each stored angle).
+cudaError_t launch_intensity_out(const float *src, double *dst, int M, long long N, const AngleMap &order,
+                                 cudaStream_t s);
 // One plane of four angles (the caller's 4q .. 4q + 3) of an array stored
 // through map, as float4 per cell: out of I into dst, or (in) from src into I.
 cudaError_t launch_plane_out(const float *I, float *dst, int q, long long N, const AngleMap &map, cudaStream_t s);
@@ -213,15 +215,21 @@ cudaError_t launch_decode_b16(const unsigned short *in, const double *E, double 
 // Scans n doubles: ORs bit 0 into *flag for a non-finite value or one below
 // `lo` (or equal to it when strict), and ORs `nzbit` for a nonzero value.
 cudaError_t launch_check(const double *x, long long n, double lo, int strict, int nzbit, int *flag, cudaStream_t s);
-// Scan of the gas fields staged as doubles (stage: rho, T, v_x, v_y, v_z,
-// sigma_a, sigma_s, N each) over cells [c0, c0 + n) into *flag (bit 0: a
+// The gas fields in doubles on the device: rho, T, sigma_a, sigma_s [N], v [3][N].
+struct FieldSrc {
+  const double *rho, *T, *v, *sa, *ss;
+};
+// Scan of the gas fields over cells [c0, c0 + n) into *flag (bit 0: a
 // value out of range, bit 1: some v != 0); with convert also the copy into
 // the context's arrays (rho, sigma_a, sigma_s, v in Real; T in double) and
 // alpha of those cells.
 template <typename Real>
-cudaError_t launch_fields_in(const double *stage, long long N, long long c0, long long n, bool convert, Real *rho,
+cudaError_t launch_fields_in(const FieldSrc &src, long long N, long long c0, long long n, bool convert, Real *rho,
                              Real *sa, Real *ss, Real *v, double *T, const CellAlpha<Real> &al, int *flag,
                              cudaStream_t s);
+// Scan of all N cells and a copy of them in stage (rho, T, v, sigma_a, sigma_s), in
+// one pass over the caller's device arrays.
+cudaError_t launch_fields_stage(const FieldSrc &src, long long N, double *stage, int *flag, cudaStream_t s);
 // alpha of N cells from their opacities.
 template <typename Real>
 cudaError_t launch_alpha(const Real *sa, const Real *ss, long long N, const CellAlpha<Real> &al, cudaStream_t s);
