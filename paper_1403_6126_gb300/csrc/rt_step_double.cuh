@@ -94,22 +94,16 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   PackedLine *s_line = reinterpret_cast<PackedLine *>(s_w + (VEL ? 3 * NBOX : 0));   // [LINES]
   const double C = a.C, invC = a.invC, dt = a.dt;
 
-  for (int m = tid; m < M; m += NT) {
-    double *t = s_tab + kTabD * m;
-    const double W = a.ang[4 * m + 3];
-    double n[3];
-    for (int d = 0; d < 3; ++d) {
-      n[d] = a.ang[4 * m + d];
-      t[d] = n[d];
-      t[4 + d] = W * n[d];
-      t[7 + d] = W * n[d] * n[d];
-      t[13 + 2 * d] = 0.5 * C * n[d] * a.dtdx[d];
-      t[14 + 2 * d] = n[d] * a.dtdx[d];
-    }
-    t[3] = W;
-    t[10] = W * n[0] * n[1];
-    t[11] = W * n[0] * n[2];
-    t[12] = W * n[1] * n[2];
+  // One entry per thread and turn: as products of three factors they cost the warp
+  // two operations for every NT entries.
+  for (int k = tid; k < kTabD * M; k += NT) {
+    const int m = k / kTabD, e = k - kTabD * m;
+    // n_i; W; W n_i; W n_i n_j; (C/2) n_d (dt/dx), n_d (dt/dx)
+    const int i = e < 3 ? e : e < 4 ? 3 : e < 7 ? e - 4 : e < 10 ? e - 7 : e < 13 ? (e == 12 ? 1 : 0) : (e - 13) >> 1;
+    const int j = e < 10 ? e - 7 : e == 10 ? 1 : 2;
+    const double *n = a.ang + 4 * m, ni = n[i], dtdx = i == 0 ? a.dtdx[0] : i == 1 ? a.dtdx[1] : a.dtdx[2];
+    const double x = e < 4 ? 1.0 : e < 13 ? n[3] : e & 1 ? 0.5 * C : 1.0;
+    s_tab[k] = x * ni * (e < 7 ? 1.0 : e < 13 ? n[j] : dtdx);
   }
 
   // ---- staged cells of this thread (see process_tile_sym) ----------------------
@@ -386,23 +380,31 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   }
 
   // ---- Step 4 solve: S, J, v.H affine in theta; scalar quartic in T ---------
-  const double v2 = vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2];
-  const double kap = A1 * invC;
-  const double Gr = v2 * Uk[0] + Uk[2], G1 = v2 * Tk[0] + Tk[2];
-  const double Ve = A1 * (C * Tk[1] + 3.0 * Tk[2]);
-  const double Ge = A1 * (C * G1 + 3.0 * (v2 * Tk[1] + Tk[3]));
-  const double Wq = Tk[0] - 4.0 * A1 * Tk[1];     // sum W (d - e) / d
-  const double rden = rcp_cubic(1.0 + kap * G1);
-  const double S0 = Gr * rden, S1 = Ge * rden;
-  const double J0 = Uk[0] - kap * S0 * Tk[0];
-  const double H0 = Uk[1] - kap * S0 * Tk[1], H1 = Ve - kap * S1 * Tk[1];
-  const double omJ1 = Wq + kap * S1 * Tk[0];   // 1 - dJ/dtheta, cancellation-free
+  // Without velocity terms vn = 0, only the sums without vn remain, and S, H and s2 vanish.
+  double v2 = 0, kap = 0, S0 = 0, S1 = 0, J0 = Uk[0], H0 = 0, H1 = 0, omJ1 = Tk[0];
+  if (VEL) {
+    v2 = vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2];
+    kap = A1 * invC;
+    const double Gr = v2 * Uk[0] + Uk[2], G1 = v2 * Tk[0] + Tk[2];
+    const double Ve = A1 * (C * Tk[1] + 3.0 * Tk[2]);
+    const double Ge = A1 * (C * G1 + 3.0 * (v2 * Tk[1] + Tk[3]));
+    const double Wq = Tk[0] - 4.0 * A1 * Tk[1];     // sum W (d - e) / d
+    const double rden = rcp_cubic(1.0 + kap * G1);
+    S0 = Gr * rden;
+    S1 = Ge * rden;
+    J0 = Uk[0] - kap * S0 * Tk[0];
+    H0 = Uk[1] - kap * S0 * Tk[1];
+    H1 = Ve - kap * S1 * Tk[1];
+    omJ1 = Wq + kap * S1 * Tk[0];   // 1 - dJ/dtheta, cancellation-free
+  }
   const double kv = rho * a.kv_per_rho;
   double T1 = T0;
   if (!a.hold_T) {
-    const double beta = a.P * C * (1.0 - v2 * invC * invC) * sa;
-    const double c0 = dt * (8.0 * kPi * a.P * sa * (H0 - S0 * invC) - 4.0 * kPi * beta * J0) - kv * T0;
-    const double c4 = dt * (2.0 * a.P * sa * (H1 - S1 * invC) + beta * omJ1);
+    const double beta = a.P * C * (VEL ? 1.0 - v2 * invC * invC : 1.0) * sa;
+    const double kin0 = VEL ? 8.0 * kPi * a.P * sa * (H0 - S0 * invC) : 0.0;
+    const double kin1 = VEL ? 2.0 * a.P * sa * (H1 - S1 * invC) : 0.0;
+    const double c0 = dt * (kin0 - 4.0 * kPi * beta * J0) - kv * T0;
+    const double c4 = dt * (kin1 + beta * omJ1);
     // the FP64 reference's iteration and stopping rule (with its default
     // options): Newton from T^n until |dT| <= newton_rtol T, then one more
     // step, at most newton_max_it steps
@@ -425,23 +427,30 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
     T1 = T;
   }
   const double T1sq = T1 * T1, th = T1sq * T1sq * (1.0 / (4.0 * kPi));
-  const double kS = kap * (S0 + th * S1);
+  double kS = 0, s1, s2 = 0, cq = 0;
+  if (VEL) {
+    kS = kap * (S0 + th * S1);
 
-  // ---- Step 5 solve: (1+B1) s1 + Bc s2 = Br,  A1 s1 + (1+Ac) s2 = Ar -------
-  // b_m = bq0 + bq1 vn + bq2 vn^2, c_m = cq vn; e_m / d_m = A1 (C + 3 vn) / d_m
-  const double bq0 = -a1 * C - a1 * v2 * invC, bq1 = 2.0 * a1, bq2 = -a1 * invC, cq = -3.0 * a1;
-  const double Bd = bq0 * Dk[0] + bq1 * Dk[1] + bq2 * Dk[2], Bdv = bq0 * Dk[1] + bq1 * Dk[2] + bq2 * Dk[3];
-  const double Ap = A1 * (C * Dk[0] + 3.0 * Dk[1]), Bp = A1 * (C * Bd + 3.0 * Bdv);
-  const double BQ = bq0 * Kk[0] + bq1 * Kk[1] + bq2 * Kk[2];
-  const double Ar = Kk[0] + th * Ap - kS * Dk[0];
-  const double Br = BQ + th * Bp - kS * Bd;
-  // 1 + sum W b / a', formed without cancellation
-  const double m11 = (1.0 - a1 * v2 * invC) * Pk[0] + a1 * Pk[1] - a1 * invC * Pk[2];
-  const double m12 = cq * (bq0 * Pk[1] + bq1 * Pk[2] + bq2 * Pk[3]);
-  const double m21 = Pk[0], m22 = 1.0 + cq * Pk[1];
-  const double rdet = rcp_cubic(m11 * m22 - m12 * m21);
-  const double s1 = (Br * m22 - m12 * Ar) * rdet;
-  const double s2 = (m11 * Ar - m21 * Br) * rdet;
+    // ---- Step 5 solve: (1+B1) s1 + Bc s2 = Br,  A1 s1 + (1+Ac) s2 = Ar -------
+    // b_m = bq0 + bq1 vn + bq2 vn^2, c_m = cq vn; e_m / d_m = A1 (C + 3 vn) / d_m
+    const double bq0 = -a1 * C - a1 * v2 * invC, bq1 = 2.0 * a1, bq2 = -a1 * invC;
+    cq = -3.0 * a1;
+    const double Bd = bq0 * Dk[0] + bq1 * Dk[1] + bq2 * Dk[2], Bdv = bq0 * Dk[1] + bq1 * Dk[2] + bq2 * Dk[3];
+    const double Ap = A1 * (C * Dk[0] + 3.0 * Dk[1]), Bp = A1 * (C * Bd + 3.0 * Bdv);
+    const double BQ = bq0 * Kk[0] + bq1 * Kk[1] + bq2 * Kk[2];
+    const double Ar = Kk[0] + th * Ap - kS * Dk[0];
+    const double Br = BQ + th * Bp - kS * Bd;
+    // 1 + sum W b / a', formed without cancellation
+    const double m11 = (1.0 - a1 * v2 * invC) * Pk[0] + a1 * Pk[1] - a1 * invC * Pk[2];
+    const double m12 = cq * (bq0 * Pk[1] + bq1 * Pk[2] + bq2 * Pk[3]);
+    const double m21 = Pk[0], m22 = 1.0 + cq * Pk[1];
+    const double rdet = rcp_cubic(m11 * m22 - m12 * m21);
+    s1 = (Br * m22 - m12 * Ar) * rdet;
+    s2 = (m11 * Ar - m21 * Br) * rdet;
+  } else {
+    // (1 + B1) s1 = Br alone, with b_m = -a1 C
+    s1 = -a1 * C * (Kk[0] + th * (A1 * C * Dk[0])) * rcp_cubic(Pk[0]);
+  }
 
   // ---- I^{n+1} over Q_m, quadrature (sec. 3) ------------------------------------
   // I = (Q + (y0 + y1 vn) / d - s1 - cq s2 vn) / a'
