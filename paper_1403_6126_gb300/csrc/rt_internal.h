@@ -120,13 +120,13 @@ cudaError_t launch_step(const StepArgs<Real> &a, int dim, bool has_v, TileShape 
 
 // The default tile of an n[0] x n[1] x n[2] grid on sms SMs: the first compiled
 // shape that fits shared memory for (dim, M, has_v), or in 1-D and 2-D the
-// smallest further one (down to 64 cells, 128 in 2-D float) that still has
-// no more tiles than there are SMs.  Such a grid runs as one CTA per SM, so a
+// smallest further one (down to 64 cells; 128 in 2-D float, 32 in 1-D double) that
+// still has no more tiles than there are SMs.  Such a grid runs as one CTA per SM, so a
 // step lasts as long as one tile and the smaller tile is the shorter one;
 // past one CTA per SM its larger halo costs more than it spreads
 // (us per step with the first shape and with the chosen one: float 1-D 512 x 8
 // angles 12.6 and 8.8, 4096 x 48 24.9 and 16.7, 2-D 64 x 48 x 24 16.0 and 14.3,
-// 128^2 x 24 16.3 and 14.6; double 512 x 8 47 and 29, 128^2 x 24 126 and 115;
+// 128^2 x 24 16.3 and 14.6; double 512 x 8 38 and 16.5, 128^2 x 24 126 and 115;
 // the other way, 256 x 128 x 80 in double, 16 x 16 377, 16 x 8 600).  3-D
 // keeps its first shape, the fastest from 24^3 up.  False if no shape fits.
 template <typename Real>

@@ -62,7 +62,7 @@ template <typename Real>
 bool choose_tile(int dim, int M, bool has_v, const int *n, int sms, TileShape *out) {
   TileShape list[16];
   const int k = shape_list<Real>(dim, list);
-  const int least = sizeof(Real) == 4 && dim == 2 ? 128 : 64;
+  const int least = sizeof(Real) == 8 && dim == 1 ? 32 : sizeof(Real) == 4 && dim == 2 ? 128 : 64;
   bool any = false;
   for (int i = 0; i < k; ++i) {
     const TileShape t = list[i];

@@ -49,12 +49,26 @@ namespace stepk {
 // xy, xz, yz), per axis C mu dt/2dx and mu dt/dx (13-18).
 constexpr int kTabD = 19;
 
+// Groups of threads per tile: each takes every GR-th round of angles of all the
+// tile's cells, and the groups add their sums up.  An FP64 instruction holds a
+// scheduler for 64 cycles whether one lane of the warp is active or all
+// (measured: 65 to 77 cycles per multiply-add at 1 to 32 lanes, one warp per scheduler), so a small grid gains
+// by more and shorter warps alone: the 1-D tile of 32 cells runs four groups,
+// a warp per scheduler, on lines of two cells.  us per step on 64-cell tiles of one group and here:
+// 512 cells x 8 angles 24.7 and 16.5, 512 x 32 68 and 31, 4096 x 48 99 and 43.
+template <int DIM, int TX, int TY, int TZ>
+constexpr int kGroupsD = DIM == 1 && TX == 32 ? 4 : 1;
+
 template <int DIM, bool VEL, int TX, int TY, int TZ>
 struct DoubleGeo {
-  using G = SymGeo<DIM, TX, TY, TZ>;
+  static constexpr int GR = kGroupsD<DIM, TX, TY, TZ>;
+  using G = SymGeo<DIM, TX, TY, TZ, (GR > 1 ? 2 : 8)>;
   static constexpr int ROUND = G::NT / G::LINES < 8 ? G::NT / G::LINES : 8;   // angles per round
+  static constexpr int SUMS = 21;   // partial sums of a group and cell
+  static_assert(GR == 1 || G::NT == 32, "a group is a warp");
   __host__ static size_t smem_bytes(int M) {
-    return sizeof(double) * (kTabD * (size_t)M + ROUND * ((VEL ? 2 : 1) * G::NBOX + G::NF) + (VEL ? 3 * G::NBOX : 0)) +
+    return sizeof(double) * (kTabD * (size_t)M + GR * ROUND * ((VEL ? 2 : 1) * G::NBOX + G::NF) +
+                             (VEL ? 3 * G::NBOX : 0) + (GR > 1 ? GR * SUMS * G::NT : 0)) +
            sizeof(double2) * G::NC + sizeof(PackedLine) * G::LINES;
   }
 };
@@ -77,26 +91,31 @@ __device__ __forceinline__ double vl_diff(double dl, double dr) {
 }
 
 template <int DIM, bool VEL, int TX, int TY, int TZ>
-__device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int tid, int tbx, int tby, int tbz,
+__device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int thread, int tbx, int tby, int tbz,
                                                unsigned char *smem_raw) {
-  using G = SymGeo<DIM, TX, TY, TZ>;
-  constexpr int NT = G::NT, ROUND = DoubleGeo<DIM, VEL, TX, TY, TZ>::ROUND, SLOTS = G::SLOTS, NBOX = G::NBOX;
+  using DG = DoubleGeo<DIM, VEL, TX, TY, TZ>;
+  using G = typename DG::G;
+  constexpr int NT = G::NT, ROUND = DG::ROUND, SLOTS = G::SLOTS, NBOX = G::NBOX, GR = DG::GR;
+  const int tid = GR > 1 ? thread % NT : thread, group = GR > 1 ? thread / NT : 0;
   const int M = a.M;
   const long long N = a.N;
   const int org[3] = {tbx * TX, tby * TY, tbz * TZ};
 
   double2 *s_fc = reinterpret_cast<double2 *>(smem_raw);        // face constants [NC]
   double *s_tab = reinterpret_cast<double *>(s_fc + G::NC);     // [M][kTabD]
-  double *s_It = s_tab + kTabD * M;                             // I~ [ROUND][NBOX]
+  double *s_all = s_tab + kTabD * M;                            // per group: I~, Delta F, IV
+  constexpr int PART = ROUND * ((VEL ? 2 : 1) * NBOX + G::NF);
+  double *s_It = s_all + group * PART;                          // I~ [ROUND][NBOX]
   double *s_F = s_It + ROUND * NBOX;                            // Delta F per axis [ROUND][NF]
   double *s_IV = s_F + ROUND * G::NF;                           // IV [ROUND][NBOX] (VEL)
-  double *s_w = s_IV + (VEL ? ROUND * NBOX : 0);                // w = 3 J v [3][NBOX] (VEL)
-  PackedLine *s_line = reinterpret_cast<PackedLine *>(s_w + (VEL ? 3 * NBOX : 0));   // [LINES]
+  double *s_w = s_all + GR * PART;                              // w = 3 J v [3][NBOX] (VEL)
+  double *s_sum = s_w + (VEL ? 3 * NBOX : 0);                   // [GR][SUMS][NT] (GR > 1)
+  PackedLine *s_line = reinterpret_cast<PackedLine *>(s_sum + (GR > 1 ? GR * DG::SUMS * NT : 0));   // [LINES]
   const double C = a.C, invC = a.invC, dt = a.dt;
 
   // One entry per thread and turn: as products of three factors they cost the warp
   // two operations for every NT entries.
-  for (int k = tid; k < kTabD * M; k += NT) {
+  for (int k = thread; k < kTabD * M; k += NT * GR) {
     const int m = k / kTabD, e = k - kTabD * m;
     // n_i; W; W n_i; W n_i n_j; (C/2) n_d (dt/dx), n_d (dt/dx)
     const int i = e < 3 ? e : e < 4 ? 3 : e < 7 ? e - 4 : e < 10 ? e - 7 : e < 13 ? (e == 12 ? 1 : 0) : (e - 13) >> 1;
@@ -130,7 +149,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
     }
     sl_box[s] = box | (code << 16);
     sl_g[s] = (int)(g[0] + (long long)a.n[0] * (g[1] + (long long)a.n[1] * g[2]));
-    if (VEL) {
+    if (VEL && group == 0) {
       const double w3 = (3.0 / (4.0 * kPi)) * a.mom_in[sl_g[s]];
       for (int d = 0; d < 3; ++d) s_w[d * NBOX + box] = w3 * a.v[d * N + sl_g[s]];
     }
@@ -143,16 +162,16 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
       for (int s = 0; s < SLOTS; ++s)
         if (m0 + k < M && used(s)) pf[k][s] = a.I_in[(long long)(m0 + k) * N + sl_g[s]];
   };
-  fetch(0);
+  fetch(group * ROUND);
 
   // ---- alpha and v of the cells -1 .. T of every axis: face constants -----------
   // alpha of each cell (per axis where the cell sides differ), kept in the I~
   // arrays meanwhile
-  double *c_al = s_It, *c_v = s_It;
+  double *c_al = s_all, *c_v = s_all;
   const bool same_dx = (DIM < 2 || a.dx[1] == a.dx[0]) && (DIM < 3 || a.dx[2] == a.dx[0]);
   for (int pass = 0; pass < (same_dx ? 1 : DIM); ++pass) {
     if (pass) __syncthreads();
-    for (int k = tid; k < G::INNER; k += NT) {
+    for (int k = thread; k < G::INNER; k += NT * GR) {
       int l[3], g[3];
       const int box = G::staged(G::inner(k), l);
       for (int d = 0; d < 3; ++d) {
@@ -163,7 +182,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
       c_al[box] = (pass == 0 ? a.alpha[0] : pass == 1 ? a.alpha[1] : a.alpha[2])[cc];
     }
     __syncthreads();
-    if (tid < G::LINES) {
+    if (thread < G::LINES) {
       Line ln{};
       const int d = G::line(tid, ln), L = d == 0 ? G::LX : d == 1 ? G::LY : G::LZ;
       if (pass == 0) s_line[tid].pack(ln);
@@ -187,10 +206,10 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
       __syncthreads();
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s)
-        if (used(s)) c_v[sl_box[s] & 0xffff] = a.v[d * N + sl_g[s]];
+        if (group == 0 && used(s)) c_v[sl_box[s] & 0xffff] = a.v[d * N + sl_g[s]];
       __syncthreads();
       const int first = d == 0 ? 0 : d == 1 ? G::NPX : G::NPX + G::NPY, np = d == 0 ? G::NPX : d == 1 ? G::NPY : G::NPZ;
-      if (tid < np) {
+      if (thread < np) {
         Line ln{};
         G::line(first + tid, ln);
         double2 *fc = s_fc + (d == 0 ? 0 : d == 1 ? G::CY : G::CZ) + tid;
@@ -245,7 +264,8 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   const int kq = tid / G::LINES, line = tid % G::LINES;
   const int axis = line < G::NPX ? 0 : DIM == 2 || line < G::NPX + G::NPY ? 1 : 2;
 #pragma unroll 1
-  for (int m0 = 0; m0 < M; m0 += ROUND) {
+  for (int mr = 0; mr < M; mr += GR * ROUND) {
+    const int m0 = mr + group * ROUND;   // the group's angles of this round
     double I0[ROUND];   // the own cell's I^n (slot 0 is the own cell)
 #pragma unroll
     for (int k = 0; k < ROUND; ++k) {
@@ -272,7 +292,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
         s_It[k * NBOX + box] = I;
       }
     }
-    fetch(m0 + ROUND);
+    fetch(m0 + GR * ROUND);
     __syncthreads();
     if (kq < ROUND && m0 + kq < M) {
       const double *t = s_tab + kTabD * (m0 + kq);
@@ -371,7 +391,30 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
       a.I_out[(long long)m * N + c] = Q;
     }
   }
-  if (!valid) return;
+  // Adds up n sums of the groups (in their order) and hands the totals to every thread.
+  auto total = [&](auto count, double *const (&x)[decltype(count)::value]) {
+    constexpr int n = decltype(count)::value;
+    static_assert(n <= DG::SUMS, "room for a group's sums");
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < n; ++i) s_sum[(group * n + i) * NT + tid] = *x[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      double t = s_sum[i * NT + tid];
+#pragma unroll
+      for (int g = 1; g < GR; ++g) t += s_sum[(g * n + i) * NT + tid];
+      *x[i] = t;
+    }
+  };
+  if constexpr (GR == 1) {
+    if (!valid) return;
+  } else if constexpr (VEL) {
+    total(IntTag<21>{}, {&Tk[0], &Tk[1], &Tk[2], &Tk[3], &Pk[0], &Pk[1], &Pk[2], &Pk[3], &Dk[0], &Dk[1], &Dk[2],
+                         &Dk[3], &Uk[0], &Uk[1], &Uk[2], &Kk[0], &Kk[1], &Kk[2], &pre[0], &pre[1], &pre[2]});
+  } else {
+    total(IntTag<6>{}, {&Ws, &Uk[0], &Kk[0], &pre[0], &pre[1], &pre[2]});
+  }
   if (!VEL) {
     Tk[0] = Ws * rd0;
     Pk[0] = Ws * ra0;
@@ -399,7 +442,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   }
   const double kv = rho * a.kv_per_rho;
   double T1 = T0;
-  if (!a.hold_T) {
+  if (!a.hold_T && (GR == 1 || valid)) {
     const double beta = a.P * C * (VEL ? 1.0 - v2 * invC * invC : 1.0) * sa;
     const double kin0 = VEL ? 8.0 * kPi * a.P * sa * (H0 - S0 * invC) : 0.0;
     const double kin1 = VEL ? 2.0 * a.P * sa * (H1 - S1 * invC) : 0.0;
@@ -423,7 +466,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
       if (extra == 0) break;
       if (extra < 0 && fabs(dT) <= rtol * T) extra = 0;
     }
-    if (it >= max_it) atomicAdd(a.status, 1);
+    if (it >= max_it && group == 0) atomicAdd(a.status, 1);
     T1 = T;
   }
   const double T1sq = T1 * T1, th = T1sq * T1sq * (1.0 / (4.0 * kPi));
@@ -457,12 +500,16 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
   const double y0 = A1 * C * th - kS, y1 = 3.0 * A1 * th, z1 = cq * s2;
   const double k0 = (y0 * rd0 - s1) * ra0;   // without velocity: I = Q / a' + k0
   double mom[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  double Qn = a.I_out[c], Qnn = a.I_out[(M > 1 ? N : 0) + c];
+  // the group's next angle, its right-hand sides read two angles ahead
+  auto after = [](int m) { return GR == 1 || (m + 1) % ROUND ? m + 1 : m + 1 + (GR - 1) * ROUND; };
+  const int first = group * ROUND;
+  auto read = [&](int m) { return (GR == 1 || valid) && m < M ? a.I_out[(long long)m * N + c] : 0.0; };
+  double Qn = read(first), Qnn = read(after(first));
 #pragma unroll 2
-  for (int m = 0; m < M; ++m) {
+  for (int m = first; m < M; m = after(m)) {
     const double Q = Qn;
     Qn = Qnn;
-    if (m + 2 < M) Qnn = a.I_out[(long long)(m + 2) * N + c];   // two angles ahead
+    Qnn = read(after(after(m)));
     const double *t = s_tab + kTabD * m;
     double I1;
     if (VEL) {
@@ -472,11 +519,34 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
     } else {
       I1 = Q * ra0 + k0;
     }
-    a.I_out[(long long)m * N + c] = I1;
+    if (GR == 1 || valid) a.I_out[(long long)m * N + c] = I1;
 #pragma unroll
     for (int i = 0; i < 10; ++i) mom[i] += t[3 + i] * I1;   // W, W n_i, W n_i n_j
   }
-  for (int i = 0; i < 10; ++i) a.mom_out[(long long)i * N + c] = 4.0 * kPi * mom[i];
+  if constexpr (GR == 1) {
+    for (int i = 0; i < 10; ++i) a.mom_out[(long long)i * N + c] = 4.0 * kPi * mom[i];
+  } else {
+    // group 0 adds up E, F and goes on to the sources, the others two of P each
+    static_assert(GR == 4, "four groups");
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 10; ++i) s_sum[(group * 10 + i) * NT + tid] = mom[i];
+    __syncthreads();
+    auto moment = [&](int i) {
+      double t = s_sum[i * NT + tid];
+#pragma unroll
+      for (int g = 1; g < GR; ++g) t += s_sum[(g * 10 + i) * NT + tid];
+      if (valid) a.mom_out[(long long)i * N + c] = 4.0 * kPi * t;
+      return t;
+    };
+    if (group > 0) {
+      moment(2 + 2 * group);
+      moment(3 + 2 * group);
+      return;
+    }
+    for (int i = 0; i < 4; ++i) mom[i] = moment(i);
+    if (!valid) return;
+  }
 
   // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
   const double kmom = -4.0 * kPi * a.P * invC;
@@ -493,7 +563,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int ti
 }
 
 template <int DIM, bool VEL, int TX, int TY, int TZ>
-__global__ void __launch_bounds__(TX * TY * TZ) step_kernel_d(const StepArgs<double> a) {
+__global__ void __launch_bounds__(TX * TY * TZ * kGroupsD<DIM, TX, TY, TZ>) step_kernel_d(const StepArgs<double> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int o = a.outer_begin;
   process_tile_d<DIM, VEL, TX, TY, TZ>(a, threadIdx.x, blockIdx.x + (DIM == 1 ? o : 0), blockIdx.y + (DIM == 2 ? o : 0),
@@ -508,7 +578,7 @@ cudaError_t launch_shape_d(const StepArgs<double> &a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   dim3 grid((a.n[0] + TX - 1) / TX, (a.n[1] + TY - 1) / TY, (a.n[2] + TZ - 1) / TZ);
   if (a.outer_count > 0) (DIM == 3 ? grid.z : DIM == 2 ? grid.y : grid.x) = a.outer_count;
-  kern<<<grid, TX * TY * TZ, sm, s>>>(a);
+  kern<<<grid, TX * TY * TZ * kGroupsD<DIM, TX, TY, TZ>, sm, s>>>(a);
   return cudaGetLastError();
 }
 

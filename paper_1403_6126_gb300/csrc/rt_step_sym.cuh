@@ -147,10 +147,10 @@ struct PackedLine {
 // kept as [position][line], x and y with one line of padding (threads that
 // read a row along x then fall on different banks), their face constants as
 // [face][line].
-template <int DIM, int TX, int TY, int TZ>
+template <int DIM, int TX, int TY, int TZ, int LMAX = 8>
 struct SymGeo {
   static constexpr int NT = TX * TY * TZ;
-  static constexpr int LX = TX < 8 ? TX : 8, LY = TY < 8 ? TY : 8, LZ = TZ;
+  static constexpr int LX = TX < LMAX ? TX : LMAX, LY = TY < LMAX ? TY : LMAX, LZ = TZ;
   static constexpr int NPX = NT / LX, NPY = DIM >= 2 ? NT / LY : 0, NPZ = DIM >= 3 ? NT / LZ : 0;
   static constexpr int LINES = NPX + NPY + NPZ;         // lines of one quad
   static constexpr int ROUND = NT / LINES < 4 ? NT / LINES : 4;   // quads per round: a line per thread at most

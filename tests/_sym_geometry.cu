@@ -26,9 +26,9 @@ static int failures = 0;
     }                                                                                                   \
   } while (0)
 
-template <int DIM, int TX, int TY, int TZ>
+template <int DIM, int TX, int TY, int TZ, int LMAX = 8>
 void check() {
-  using G = SymGeo<DIM, TX, TY, TZ>;
+  using G = SymGeo<DIM, TX, TY, TZ, LMAX>;
   auto key = [](const int l[3]) { return (l[0] + 100) + 1000 * ((l[1] + 100) + 1000 * (l[2] + 100)); };
   const int T[3] = {TX, TY, TZ};
   std::map<int, int> place;
@@ -104,6 +104,7 @@ int main() {
   check<1, 128, 1, 1>();
   check<1, 64, 1, 1>();
   check<1, 32, 1, 1>();
+  check<1, 32, 1, 1, 2>();
   if (failures == 0) std::printf("OK\n");
   return failures == 0 ? 0 : 1;
 }

@@ -32,7 +32,9 @@ def _context(name, kw, precision):
 @pytest.mark.parametrize("name,kw,precision,tile,first", [
     ("slab1d", dict(n=64 * SMS, steps=0), "fp32", (64, 1, 1), (512, 1, 1)),
     ("slab1d", dict(n=64 * SMS + 1, steps=0), "fp32", (128, 1, 1), (512, 1, 1)),
-    ("slab1d", dict(n=33, steps=0), "fp64", (64, 1, 1), (256, 1, 1)),
+    ("slab1d", dict(n=33, steps=0), "fp64", (32, 1, 1), (256, 1, 1)),
+    ("slab1d", dict(n=32 * SMS, M=48, steps=0), "fp64", (32, 1, 1), (256, 1, 1)),
+    ("slab1d", dict(n=32 * SMS + 1, steps=0), "fp64", (64, 1, 1), (256, 1, 1)),
     ("slab1d", dict(n=128 * SMS + 1, steps=0), "fp64", (256, 1, 1), (256, 1, 1)),
     ("shadow2d", dict(nx=16 * SMS, ny=8, angles="s4", steps=0), "fp32", (16, 8, 1), (32, 16, 1)),
     ("shadow2d", dict(nx=16 * SMS + 1, ny=16, angles="s4", steps=0), "fp32", (16, 16, 1), (32, 16, 1)),
@@ -92,3 +94,35 @@ def test_coupled_step_cut_in_small_tiles(name, kw, precision):
         np.testing.assert_array_equal(np.asarray(x).reshape(-1), np.asarray(y).reshape(-1))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n,M", [(1, 1), (31, 2), (33, 7), (64, 8), (65, 9), (100, 48)])
+@pytest.mark.parametrize("moving", [False, True])
+def test_grouped_double_tile_matches_plain_tile(n, M, moving):
+    # the 32-cell tile shares its angles out among four groups of threads
+    wl = dict(wlmod.slab1d(n=n, steps=0))
+    wl.update(hold_T=False, estimate_v=moving)
+    rng = np.random.default_rng(n + M)
+    v = np.zeros((3, n))
+    if moving:
+        v[:, n // 3:] = 0.1 * wl["C"] * (rng.random((3, n - n // 3)) - 0.5)
+    nn = rng.normal(size=(M, 3))
+    nn = np.ascontiguousarray(nn / np.sqrt((nn * nn).sum(1, keepdims=True)))
+    w = rng.random(M) + 0.5
+    w = w / w.sum()
+    I = rng.random((M, n))
+    out = []
+    for tile in ((32, 1, 1), (64, 1, 1)):
+        ctx = gpu_context(wl, nn, w, "fp64")
+        ctx.set_tile(*tile)
+        ctx.set_intensity(I)
+        ctx.set_material(wl["rho"], wl["T"], v, wl["sa"], wl["ss"])
+        for _ in range(3):
+            ctx.step(0.0)
+        ctx.sync()
+        out.append([ctx.intensity(), *ctx.moments(), *ctx.sources()])
+        ctx.close()
+    scale = np.abs(out[1][1]).max()     # E: momentum and energy sources are differences of terms of P E / C, P E
+    for k, (a, b) in enumerate(zip(*out)):
+        tol = 1e-11 * max(np.abs(b).max(), scale)
+        assert np.abs(a - b).max() <= tol, k
