@@ -31,6 +31,7 @@ struct rt_ctx {
   bool has_v = false, material_set = false, intensity_set = false;
   rtg::TileShape tile{0, 0, 0};
   int dev = 0, sms = 0;   // the context's device and its SMs
+  void *block = nullptr;  // the device allocation that holds every array below
   // device state (Real = double or float)
   void *I[2] = {nullptr, nullptr};
   double *mom[2] = {nullptr, nullptr};   // E, F, P [10][N], double for every precision
@@ -68,6 +69,8 @@ namespace rtg {
 // Device allocation of the library: cudaMalloc, unless rt_fault_inject has
 // armed a failure for this allocation.
 cudaError_t device_alloc(void **p, size_t bytes);
+// Counts one allocation against rt_fault_inject; whether it is the one to fail.
+bool allocation_fails();
 // NVTX range over an entry point (free when no profiler is attached).
 struct Range {
   explicit Range(const char *name) { nvtxRangePushA(name); }
