@@ -147,7 +147,16 @@ struct PackedLine {
 // kept as [position][line], x and y with one line of padding (threads that
 // read a row along x then fall on different banks), their face constants as
 // [face][line].
-template <int DIM, int TX, int TY, int TZ, int LMAX = 8>
+//
+// Lines of eight cells, or of four in a 3-D tile of 128 cells: its lines along y
+// and z are that short already, and the eight-cell ones along x kept the other
+// threads waiting (8x4x4, us per step: 96 x 80 x 72 x 24 angles 211 -> 162, 75 x 50 x 61 x
+// 48 without velocity 134 -> 99, 128^3 x 80 2066 -> 1363; the larger tiles, with
+// a line for every thread, lose by it: 8x8x4 1261 -> 1381).
+template <int DIM, int TX, int TY, int TZ>
+constexpr int kLineMax = DIM == 3 && TX * TY * TZ == 128 ? 4 : 8;
+
+template <int DIM, int TX, int TY, int TZ, int LMAX = kLineMax<DIM, TX, TY, TZ>>
 struct SymGeo {
   static constexpr int NT = TX * TY * TZ;
   static constexpr int LX = TX < LMAX ? TX : LMAX, LY = TY < LMAX ? TY : LMAX, LZ = TZ;

@@ -105,6 +105,7 @@ int main() {
   check<1, 64, 1, 1>();
   check<1, 32, 1, 1>();
   check<1, 32, 1, 1, 2>();
+  check<3, 8, 4, 4, 4>();
   if (failures == 0) std::printf("OK\n");
   return failures == 0 ? 0 : 1;
 }
