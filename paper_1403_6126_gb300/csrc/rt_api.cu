@@ -280,6 +280,29 @@ rt_status delivered(rt_ctx *c) {
   return RT_OK;
 }
 
+// Up to three device arrays to the caller's (null: not wanted).  Into device
+// arrays that a kernel may write they go by one launch: a copy costs the host
+// about as much, and small problems are many (24 steps of 512 problems and their
+// moments 23.4 -> 19.2 ms, gas loop 233 -> 228 us).
+rt_status deliver_fields(rt_ctx *c, const rtg::FieldsOut &want) {
+  rtg::FieldsOut f = want;
+  int count = 0;
+  bool direct = true;
+  for (int i = 0; i < 3; ++i) {
+    if (!f.dst[i]) f.n[i] = 0;
+    count += f.dst[i] != nullptr;
+    direct = direct && (!f.dst[i] || in_place(c, f.dst[i]));
+  }
+  if (direct && count > 1) {
+    RT_CUDA(rtg::launch_fields_out(f, c->stream));
+    return RT_OK;
+  }
+  rt_status st;
+  for (int i = 0; i < 3; ++i)
+    if (f.dst[i] && (st = deliver_async(c, f.src[i], f.dst[i], f.n[i])) != RT_OK) return st;
+  return delivered(c);
+}
+
 // Copies n doubles from the device buffer src to the caller (host: waits).
 rt_status deliver(rt_ctx *c, const double *src, double *dst, long long n) {
   rt_status st = deliver_async(c, src, dst, n);
@@ -1023,11 +1046,7 @@ rt_status rt_moments(rt_ctx *c, double *E, double *F, double *P) {
   if (!c->intensity_set) return fail(RT_E_STATE, "rt_moments: no intensity yet");
   const long long N = c->N;
   const double *mom = c->mom[c->cur];
-  rt_status st;
-  if (E && (st = deliver_async(c, mom, E, N)) != RT_OK) return st;
-  if (F && (st = deliver_async(c, mom + N, F, 3 * N)) != RT_OK) return st;
-  if (P && (st = deliver_async(c, mom + 4 * N, P, 6 * N)) != RT_OK) return st;
-  return delivered(c);
+  return deliver_fields(c, {{mom, mom + N, mom + 4 * N}, {E, F, P}, {N, 3 * N, 6 * N}});
 }
 
 rt_status rt_eddington(rt_ctx *c, double *f) {
@@ -1045,12 +1064,8 @@ rt_status rt_sources(rt_ctx *c, double *dE_gas, double *dMom, double *T_new) {
   rtg::Range nvtx_range("rt_sources");
   if (!c) return fail(RT_E_INVALID, "rt_sources: NULL context");
   const long long N = c->N;
-  rt_status st;
-  // the energy source and T are double on the device: copied out directly
-  if (dE_gas && (st = deliver_async(c, c->dEgas, dE_gas, N)) != RT_OK) return st;
-  if (dMom && (st = deliver_async(c, c->dMom, dMom, 3 * N)) != RT_OK) return st;
-  if (T_new && (st = deliver_async(c, c->T, T_new, N)) != RT_OK) return st;
-  return delivered(c);
+  // all double on the device: copied out directly
+  return deliver_fields(c, {{c->dEgas, c->dMom, c->T}, {dE_gas, dMom, T_new}, {N, 3 * N, N}});
 }
 
 rt_status rt_step_coupled(rt_ctx *c, double dt, const double *rho, const double *T, const double *v,

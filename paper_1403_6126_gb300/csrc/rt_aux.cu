@@ -2,6 +2,7 @@
 // isotropic equilibrium intensity, the sec. 3 quadrature of a given field,
 // and input scans.  All grid-stride, sized as a multiple of the SM count.
 #include <cuda_bf16.h>
+#include <algorithm>
 #include <math.h>
 
 #include "rt_aux.cuh"
@@ -86,6 +87,15 @@ __global__ void intensity_out_kernel(const float4 *__restrict__ I, double *__res
     if (left > 2) __stcs(out[2] + c, widen(x.z));
     if (left > 3) __stcs(out[3] + c, widen(x.w));
   }
+}
+
+// Three arrays of doubles to the caller's, blockIdx.y = which.
+__global__ void fields_out_kernel(const FieldsOut f) {
+  const double *src = blockIdx.y == 0 ? f.src[0] : blockIdx.y == 1 ? f.src[1] : f.src[2];
+  double *dst = blockIdx.y == 0 ? f.dst[0] : blockIdx.y == 1 ? f.dst[1] : f.dst[2];
+  const long long n = blockIdx.y == 0 ? f.n[0] : blockIdx.y == 1 ? f.n[1] : f.n[2];
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    dst[i] = src[i];
 }
 
 // The caller's angles 4q .. 4q + 3 of every cell as one float4 plane.
@@ -299,6 +309,13 @@ cudaError_t launch_intensity_out(const float *src, double *dst, int M, long long
                                  cudaStream_t s) {
   const dim3 grid(grid_for(N, 256), (M + 3) / 4);
   intensity_out_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4 *>(src), dst, M, N, order);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fields_out(const FieldsOut &f, cudaStream_t s) {
+  const long long n = std::max(f.n[0], std::max(f.n[1], f.n[2]));
+  if (n <= 0) return cudaSuccess;
+  fields_out_kernel<<<dim3(grid_for(n, 256), 3), 256, 0, s>>>(f);
   return cudaGetLastError();
 }
 

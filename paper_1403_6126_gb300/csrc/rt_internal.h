@@ -196,6 +196,13 @@ cudaError_t launch_quad_in(const double *src, float *dst, long long off, long lo
                            cudaStream_t s);
 cudaError_t launch_quad_out(const float *src, double *dst, long long off, long long n, long long N, const AngleMap &map,
                             cudaStream_t s);
+// Up to three arrays of doubles (n = 0: none) in one launch.
+struct FieldsOut {
+  const double *src[3];
+  double *dst[3];
+  long long n[3];
+};
+cudaError_t launch_fields_out(const FieldsOut &f, cudaStream_t s);
 // Every angle of the quad layout to the caller's [M][N] doubles (order.slot: the
 // caller's index of each stored angle).
 cudaError_t launch_intensity_out(const float *src, double *dst, int M, long long N, const AngleMap &order,

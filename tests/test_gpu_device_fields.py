@@ -109,3 +109,29 @@ def test_fields_from_device_arrays(precision, shape):
     np.testing.assert_array_equal(other.intensity(), host.intensity())
     for c in (dev, host, other):
         c.close()
+
+
+@pytest.mark.parametrize("want", [(1, 1, 1), (1, 0, 1), (0, 1, 0), (0, 0, 0)])
+@pytest.mark.parametrize("off", [0, 4])
+def test_moments_and_sources_to_device_arrays(want, off):
+    n, w = _angles("s4")
+    wl, dev, host = _pair("box3d", n, w, "fp32", dict(n=7, angles="s4", steps=0))
+    N = int(np.prod(wl["shape"]))
+    f = [np.ascontiguousarray(wl[k]).reshape(-1) for k in ("rho", "T", "v", "sa", "ss")]
+    dev.set_material(*[torch.tensor(x, dtype=torch.float64, device="cuda") for x in f])
+    host.set_material(*f)
+    for c in (dev, host):
+        c.step(0.0)
+        c.sync()
+    for call, sizes, ref in ((rt.lib().rt_moments, (1, 3, 6), host.moments()), (rt.lib().rt_sources, (1, 3, 1), host.sources())):
+        raw = [torch.zeros(8 * k * N + 8, dtype=torch.uint8, device="cuda") for k in sizes]
+        assert call(dev.ctx, *[r.data_ptr() + off if use else None for r, use in zip(raw, want)]) == rt.RT_OK
+        torch.cuda.synchronize()
+        for r, k, use, x in zip(raw, sizes, want, ref):
+            got = r.cpu().numpy()
+            if use:
+                np.testing.assert_array_equal(got[off:off + 8 * k * N].copy().view(np.float64), np.asarray(x).reshape(-1))
+            else:
+                assert not got.any()
+    dev.close()
+    host.close()
