@@ -30,10 +30,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 PROFILE = os.path.join(ROOT, "profiles", "step_kernel_box3d.md")
-# sources of the float step kernel (the quad kernel, the packed-FP32 helpers of
-# the pair kernel it includes, and the tile geometry)
+# sources of the float step kernel (the kernel of opposite pairs, the quad kernel
+# whose per-cell parts it uses, the packed-FP32 helpers and the tile geometry)
 KERNEL_SRCS = [os.path.join(ROOT, "paper_1403_6126_gb300", "csrc", f)
-               for f in ("rt_step_quad.cuh", "rt_step_pair.cuh", "rt_step_kernel.cuh")]
+               for f in ("rt_step_sym.cuh", "rt_step_quad.cuh", "rt_step_pair.cuh", "rt_step_kernel.cuh")]
 NOMINAL_HBM_GBS = 8000.0
 
 
@@ -374,9 +374,9 @@ def run_gpu(args):
                 "traffic": traffic, "peak_source": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else "fallback 6.8 TB/s",
                 "frac_of_nominal_8tbs": achieved / NOMINAL_HBM_GBS,
                 "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": avg_launch_s * 1e3,
-                "kernel": ("step_kernel_q<%d,%s,%d,%d,%d>" % ((wl["dim"], "true" if velocity else "false") + tile)
-                           if rs == 4 else "step_kernel<double,%d,%s,%d,%d,%d>"
-                           % ((wl["dim"], "true" if velocity else "false") + tile)),
+                "kernel": ("step_kernel_%s<%d,%s,%d,%d,%d>"
+                           % (("d" if rs == 8 else "sym" if wl["dim"] > 1 else "q", wl["dim"],
+                               "true" if velocity else "false") + tile)),
                 "tile": "%dx%dx%d" % tile, "autotune": tuned}
 
     # end to end through the C ABI with pinned host buffers: per step the gas

@@ -175,12 +175,13 @@ rt_status rt_set_intensity(rt_ctx *ctx, const double *I);
 rt_status rt_set_inflow(rt_ctx *ctx, int axis, int side, const double *I_ghost);
 
 /* Tile of cells one CTA of the step kernel owns (tx x ty x tz, one thread
- * per cell; ty = 1 for 1-D, tz = 1 below 3-D).  (0, 0, 0) restores the
- * default choice.  RT_E_INVALID when the shape is not one of the compiled
+ * per cell, four in the 32-cell 1-D double tile; ty = 1 for 1-D, tz = 1 below
+ * 3-D).  (0, 0, 0) restores the default choice, which follows the grid size.  RT_E_INVALID when the shape is not one of the compiled
  * shapes or exceeds the 227 KB of shared memory (which grows with the angle
  * count).  Float results do not depend on the tile (bitwise); double
- * results may differ in the last bit, as the compiler fuses multiply-adds
- * differently per tile shape.  The paper has no counterpart (its code runs
+ * results may differ by rounding, as the compiler fuses multiply-adds
+ * differently per tile shape and the 32-cell 1-D tile adds its angles up in
+ * groups.  The paper has no counterpart (its code runs
  * on CPUs). */
 rt_status rt_set_tile(rt_ctx *ctx, int tx, int ty, int tz);
 rt_status rt_get_tile(const rt_ctx *ctx, int *tx, int *ty, int *tz);
@@ -313,11 +314,11 @@ rt_status rt_batch_step(rt_batch *b, int nsteps);
 /* Tile-set autotuner of the persistent kernel.  Three variants are
  * compiled: 512, 256 and 128 threads per CTA (tiles 512 / 32x16 / 16x8x4,
  * 256 / 16x16 / 8x8x4 and 128 / 16x8 / 8x4x4 cells for 1-D / 2-D / 3-D
- * members).  Times trial_steps (>= 1, after one untimed step) of each on the
- * batch's stream and keeps the fastest for later rt_batch_step calls.  The
- * members' state is restored afterwards (bitwise).  ms (may be NULL)
- * receives the three times in the order above, *chosen (may be NULL) the
- * index kept.  Waits for the stream. */
+ * members); the second is the default.  Times trial_steps (>= 1, after one
+ * untimed step) of each on the batch's stream and keeps the fastest for later
+ * rt_batch_step calls.  The members' state is restored afterwards (bitwise).
+ * ms (may be NULL) receives the three times in the order above, *chosen (may
+ * be NULL) the index kept.  Waits for the stream. */
 rt_status rt_batch_autotune(rt_batch *b, int trial_steps, double *ms, int *chosen);
 /* Frees the batch (not its contexts).  NULL is ignored. */
 void rt_batch_destroy(rt_batch *b);

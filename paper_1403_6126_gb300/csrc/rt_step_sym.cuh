@@ -33,11 +33,11 @@
 //    term per pair.
 //
 // What bounds it: issue and latency together.  At 96^3 cells x 80 angles (8x8x4
-// tile, two CTAs of 256 threads at 125 registers) it issues 175 thread
+// tile, two CTAs of 256 threads at 125 registers) it issues 173 thread
 // instructions per cell-angle (the quad kernel 197) at 57 % of the issue rate
 // (48 %), FMA pipe 42 %, shared-memory wavefronts 24 per cell and quad (48),
 // DRAM 0.80 GB for 0.57 GB of intensities: 0.545 ms against 0.726 ms; 128^3 x
-// 80: 1.29 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
+// 80: 1.26 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
 // per SM, with the long x and y lines in one phase and the short z lines in
 // the next (0.77: 12 warps); one pair per thread, two threads per cell, 64
 // registers (0.76: 32 warps, but twice the instructions without the packed
@@ -150,8 +150,8 @@ struct PackedLine {
 //
 // Lines of eight cells, or of four in a 3-D tile of 128 cells: its lines along y
 // and z are that short already, and the eight-cell ones along x kept the other
-// threads waiting (8x4x4, us per step: 96 x 80 x 72 x 24 angles 211 -> 162, 75 x 50 x 61 x
-// 48 without velocity 134 -> 99, 128^3 x 80 2066 -> 1363; the larger tiles, with
+// threads waiting (8x4x4, us per step: 96 x 80 x 72 x 24 angles 211 -> 162,
+// 75 x 50 x 61 x 48 without velocity 134 -> 99, 128^3 x 80 2066 -> 1363; the larger tiles, with
 // a line for every thread, lose by it: 8x8x4 1261 -> 1381).
 template <int DIM, int TX, int TY, int TZ>
 constexpr int kLineMax = DIM == 3 && TX * TY * TZ == 128 ? 4 : 8;
@@ -537,9 +537,9 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
   {
     // every load before the first store to shared memory: one latency
     // (in 3-D alpha comes with the context's fields: gas loop of 96 x 80 x 72 x 24
-    // angles 264 -> 257 us; in 2-D, where one CTA per SM waits for every load, forming it
-    // here is faster, 866 against 900 us for 40 steps of 128^2 x 24: sa and ss are then
-    // in L1 when the cell's own fields are read)
+    // angles 264 -> 257 us; in 2-D, where a grid is a wave of CTAs that all wait for
+    // their loads, forming it here is faster, 866 against 900 us for 20 steps of
+    // 256^2 x 80: sa and ss are then in L1 when the cell's own fields are read)
     constexpr bool KEPT = DIM == 3 && !GATHER;
     float st[SLOTS], al[SLOTS][3], v[SLOTS][3];
     double E[SLOTS];
