@@ -13,7 +13,6 @@ from paper_1403_6126_gb300 import workloads as wlmod
 from _helpers import gpu_context, initial_state, rel_err
 from test_zz_no_alloc import test_noalloc_step_equals_rt_step as noalloc_equals_rt_step
 
-noalloc_equals_rt_step.__test__ = False
 pytestmark = pytest.mark.gpu
 SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 152
 
