@@ -329,7 +329,10 @@ __device__ __forceinline__ CellSolve solve_cell(const StepArgs<float> &a, const 
       const float T = T0f + d;
       const float f = fmaf(kvf, d, fmaf(c4, d * fmaf(d, fmaf(d, p1 + d, p2), p3), cc));
       const float fp = fmaf(4.0f * c4, T * T * T, kvf);
-      float dn = d - __fdividef(f, fp);   // the next iterate corrects its last bits
+      // the fast quotient, whose last bits the next iterate corrects, where it is
+      // defined: divisors of magnitude 2^-126 to 2^126
+      const float m = fabsf(fp);
+      float dn = d - (m >= 0x1p-126f && m <= 0x1p126f ? __fdividef(f, fp) : f / fp);
       if (!(T0f + dn > 0.0f)) dn = 0.5f * T - T0f;
       const float step = dn - d;
       d = dn;

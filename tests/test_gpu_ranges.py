@@ -1,0 +1,47 @@
+"""Accepted inputs near the ends of the number range, where a reciprocal or a
+fast quotient is not defined although the division it stands for is."""
+import numpy as np
+import pytest
+
+import oracle
+
+from _helpers import gpu_context, rel_err, run_both
+
+pytestmark = pytest.mark.gpu
+
+P = 0
+
+
+def _uniform(shape, rho, prat, sigma, T):
+    N = int(np.prod(shape))
+    dim = 3 if shape[0] > 1 else 2 if shape[1] > 1 else 1
+    return dict(name="uniform", shape=shape, dim=dim, lo=(0.0, 0.0, 0.0), hi=(1.0, 1.0, 1.0), bc=((P, P),) * 3, C=10.0, P=prat,
+                gamma=5.0 / 3.0, R=1.0, cfl=0.4, hold_T=False, estimate_v=False, steps=0, precision="fp32",
+                rho=np.full(N, rho), T=np.full(N, T), v=np.zeros((3, N)), sa=np.full(N, sigma), ss=np.zeros(N),
+                I0="isotropic_quarter_pi", inflow={}, angles="s4")
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 40), (1, 9, 12), (5, 4, 9)])
+def test_float_temperature_solve_at_a_large_heat_capacity(shape):
+    # rho R / (gamma - 1) = 1.5e38, above 2^126: the gas cools by a part in a
+    # thousand or more, as in the oracle
+    wl = _uniform(shape, 1e38, 1e35, 1.0, 3.2)
+    n, w = oracle.angles.by_name("s4")
+    g, o = run_both(wl, 3, "fp32", n=np.ascontiguousarray(n), w=np.ascontiguousarray(w))
+    assert o["T"].max() < 3.2 - 1e-3
+    assert rel_err(g["T"], o["T"]) <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 40), (1, 9, 12), (5, 4, 9)])
+def test_float_temperature_solve_at_a_subnormal_heat_capacity(shape):
+    # without opacity nothing heats the gas: T stays as it is, and no cell fails
+    wl = _uniform(shape, 1e-39, 1.0, 0.0, 1.0)
+    n, w = oracle.angles.by_name("s4")
+    ctx = gpu_context(wl, np.ascontiguousarray(n), np.ascontiguousarray(w), "fp32")
+    ctx.set_intensity(np.full((len(w), wl["rho"].size), 1.0 / (4 * np.pi)))
+    ctx.set_material(wl["rho"], wl["T"], wl["v"], wl["sa"], wl["ss"])
+    for _ in range(3):
+        ctx.step(0.0)
+    ctx.sync()
+    np.testing.assert_array_equal(ctx.sources()[2].reshape(-1), wl["T"])
+    ctx.close()
