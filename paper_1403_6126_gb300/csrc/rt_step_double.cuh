@@ -77,15 +77,32 @@ struct DoubleGeo {
   }
 };
 
-// 1/x by one cubic step from the hardware's approximation (relative error e
-// below 2^-19): r (1 + e + e^2) leaves e^3 below 2^-57, so the result is within
-// one unit in the last place.  NaN for x = 0.
-__device__ __forceinline__ double rcp_cubic(double x) {
+// 1/x by one step of the cubically convergent hyperpower iteration r (1 + e + e^2),
+// e = 1 - x r (M. Altman, Pacific J. Math. 10 (1960) 1107), from the hardware's
+// approximation: its relative error is below 2^-19 where x is a normal number
+// below 2^1022 in magnitude, so e^3 is below 2^-57 and the result within one unit
+// in the last place (1.0 / x is within half of one).  Beyond that range,
+// NaN for zero, subnormal and infinite x, 0 from 2^1022 on.
+__device__ __forceinline__ double rcp_seed(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ double rcp_cubic(double x) {
+  const double r = rcp_seed(x);
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
+
+// Whether rcp_cubic(x) is 1/x: |x| at least 2^-1022 and below 2^1022 (in integers,
+// off the FP64 pipe).
+__device__ __forceinline__ bool rcp_range(double x) {
+  return (unsigned)(__double2hiint(x) & 0x7ff00000) - 0x00100000u < 0x7fc00000u;
+}
+
+// 1/x and n/x of every x.
+__device__ __forceinline__ double rcp_any(double x) { return rcp_range(x) ? rcp_cubic(x) : 1.0 / x; }
+__device__ __forceinline__ double div_any(double n, double x) { return rcp_range(x) ? n * rcp_cubic(x) : n / x; }
 
 // Half van Leer slope from the one-sided differences (see vl_half).
 __device__ __forceinline__ double vl_diff(double dl, double dr) {
@@ -253,14 +270,14 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
           const double Fd = a.mom_in[(1 + d) * N + c], Pdd = a.mom_in[(4 + d) * N + c];
           const double num = rho * vin[d] + h * (C * rho * vin[d] + a.P * Fd);
           const double den = rho + h * (C * rho + a.P * (E + Pdd) * invC);
-          vt[d] = num * rcp_cubic(den);
+          vt[d] = div_any(num, den);
         }
       }
     }
   }
   const bool scat = ss > sa;
   const double A0 = 1.0 + dt * C * sa, A1 = dt * sa, a0 = 1.0 + dt * C * ss, a1 = dt * ss;
-  const double rd0 = VEL ? 0.0 : rcp_cubic(A0), ra0 = VEL ? 0.0 : rcp_cubic(a0);
+  const double rd0 = VEL ? 0.0 : rcp_any(A0), ra0 = VEL ? 0.0 : rcp_any(a0);
 
   // ---- transport, Q_m and the angle sums: ROUND angles per two barriers -------------
   double Tk[4] = {0, 0, 0, 0}, Pk[4] = {0, 0, 0, 0}, Dk[4] = {0, 0, 0, 0};
@@ -375,7 +392,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
       double Q;
       if (VEL) {
         const double vn = t[0] * vt[0] + t[1] * vt[1] + t[2] * vt[2];
-        const double rd = rcp_cubic(A0 - A1 * vn), ra = rcp_cubic(a0 - a1 * vn);
+        const double rd = rcp_any(A0 - A1 * vn), ra = rcp_any(a0 - a1 * vn);
         const double u = r * rd;
         Q = scat ? u + dF : u;
         const double z = Q * ra, pd = ra * rd, y1 = W * vn, y2 = y1 * vn, y3 = y2 * vn;
@@ -436,9 +453,9 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
     const double Ve = A1 * (C * Tk[1] + 3.0 * Tk[2]);
     const double Ge = A1 * (C * G1 + 3.0 * (v2 * Tk[1] + Tk[3]));
     const double Wq = Tk[0] - 4.0 * A1 * Tk[1];     // sum W (d - e) / d
-    const double rden = rcp_cubic(1.0 + kap * G1);
-    S0 = Gr * rden;
-    S1 = Ge * rden;
+    const double den = 1.0 + kap * G1;
+    S0 = div_any(Gr, den);
+    S1 = div_any(Ge, den);
     J0 = Uk[0] - kap * S0 * Tk[0];
     H0 = Uk[1] - kap * S0 * Tk[1];
     H1 = Ve - kap * S1 * Tk[1];
@@ -463,7 +480,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
       const double T3 = T * T * T;
       const double f = c4 * T3 * T + kv * T + c0;
       const double fp = 4.0 * c4 * T3 + kv;
-      double Tn = T - f * rcp_cubic(fp);
+      double Tn = T - div_any(f, fp);
       if (!(Tn > 0)) Tn = 0.5 * T;
       const double dT = Tn - T;
       T = Tn;
@@ -491,12 +508,12 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
     const double m11 = (1.0 - a1 * v2 * invC) * Pk[0] + a1 * Pk[1] - a1 * invC * Pk[2];
     const double m12 = cq * (bq0 * Pk[1] + bq1 * Pk[2] + bq2 * Pk[3]);
     const double m21 = Pk[0], m22 = 1.0 + cq * Pk[1];
-    const double rdet = rcp_cubic(m11 * m22 - m12 * m21);
-    s1 = (Br * m22 - m12 * Ar) * rdet;
-    s2 = (m11 * Ar - m21 * Br) * rdet;
+    const double det = m11 * m22 - m12 * m21;
+    s1 = div_any(Br * m22 - m12 * Ar, det);
+    s2 = div_any(m11 * Ar - m21 * Br, det);
   } else {
     // (1 + B1) s1 = Br alone, with b_m = -a1 C
-    s1 = -a1 * C * (Kk[0] + th * (A1 * C * Dk[0])) * rcp_cubic(Pk[0]);
+    s1 = div_any(-a1 * C * (Kk[0] + th * (A1 * C * Dk[0])), Pk[0]);
   }
 
   // ---- I^{n+1} over Q_m, quadrature (sec. 3) ------------------------------------
@@ -518,7 +535,7 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
     double I1;
     if (VEL) {
       const double vn = t[0] * vt[0] + t[1] * vt[1] + t[2] * vt[2];
-      const double rd = rcp_cubic(A0 - A1 * vn), ra = rcp_cubic(a0 - a1 * vn);
+      const double rd = rcp_any(A0 - A1 * vn), ra = rcp_any(a0 - a1 * vn);
       I1 = (Q + rd * (y0 + y1 * vn) - s1 - z1 * vn) * ra;
     } else {
       I1 = Q * ra0 + k0;
@@ -554,13 +571,12 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
 
   // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
   const double kmom = -4.0 * kPi * a.P * invC;
-  const double r2rho = 0.5 * rcp_cubic(rho);
   double dEK = 0;
   for (int i = 0; i < 3; ++i) {
     const double dmom = kmom * (mom[1 + i] - pre[i]);
     a.dMom[i * N + c] = dmom;
     const double m0 = rho * vin[i];
-    dEK += ((m0 + dmom) * (m0 + dmom) - m0 * m0) * r2rho;
+    dEK += div_any((m0 + dmom) * (m0 + dmom) - m0 * m0, 2.0 * rho);
   }
   a.T_out[c] = T1;
   a.dEgas[c] = kv * (T1 - T0) + dEK;

@@ -45,3 +45,24 @@ def test_float_temperature_solve_at_a_subnormal_heat_capacity(shape):
     ctx.sync()
     np.testing.assert_array_equal(ctx.sources()[2].reshape(-1), wl["T"])
     ctx.close()
+
+
+@pytest.mark.parametrize("moving", [False, True])
+@pytest.mark.parametrize("shape", [(1, 1, 40), (1, 1, 20000), (1, 9, 12), (5, 4, 9)])
+def test_double_step_at_a_subnormal_density(shape, moving):
+    # without opacity nothing acts on the gas: T stays, the sources are zero
+    wl = _uniform(shape, 1e-310, 1.0, 0.0, 1.0)
+    wl.update(estimate_v=moving, v=np.full_like(wl["v"], 0.5 * moving))
+    n, w = oracle.angles.by_name("s4")
+    n, w = np.ascontiguousarray(n), np.ascontiguousarray(w)
+    ctx = gpu_context(wl, n, w, "fp64")
+    ctx.set_intensity(np.random.default_rng(4).random((len(w), wl["rho"].size)))
+    ctx.set_material(wl["rho"], wl["T"], wl["v"], wl["sa"], wl["ss"])
+    for _ in range(3):
+        ctx.step(0.0)
+    ctx.sync()
+    dE, dM, T = ctx.sources()
+    np.testing.assert_array_equal(T.reshape(-1), wl["T"])
+    assert not np.asarray(dE).any() and not np.asarray(dM).any()
+    assert np.isfinite(ctx.intensity()).all()
+    ctx.close()
