@@ -104,11 +104,13 @@ __device__ __forceinline__ bool rcp_range(double x) {
 __device__ __forceinline__ double rcp_any(double x) { return rcp_range(x) ? rcp_cubic(x) : 1.0 / x; }
 __device__ __forceinline__ double div_any(double n, double x) { return rcp_range(x) ? n * rcp_cubic(x) : n / x; }
 
-// Half van Leer slope from the one-sided differences (see vl_half).
+// Half van Leer slope from the one-sided differences (see vl_half2).  Their product
+// is tested on its bit pattern, off the FP64 pipe: positive up to infinity, which
+// a NaN is not.  Where it is, |dl + dr| is at least 2^-537.
 __device__ __forceinline__ double vl_diff(double dl, double dr) {
   const double pr = dl * dr;
   const double h = pr * rcp_cubic(dl + dr);
-  return __double2hiint(pr) > 0 ? h : 0.0;
+  return (unsigned long long)__double_as_longlong(pr) - 1 < 0x7ff0000000000000ull ? h : 0.0;
 }
 
 template <int DIM, bool VEL, int TX, int TY, int TZ>
