@@ -573,12 +573,19 @@ __device__ __forceinline__ void process_tile_d(const StepArgs<double> &a, int th
 
   // ---- gas sources (sec. 4.3: Delta E_T, eqs. momentumchange, kinetichange)
   const double kmom = -4.0 * kPi * a.P * invC;
-  double dEK = 0;
+  double dEK = 0, work[3];   // 2 rho times the work on each component
   for (int i = 0; i < 3; ++i) {
     const double dmom = kmom * (mom[1 + i] - pre[i]);
     a.dMom[i * N + c] = dmom;
     const double m0 = rho * vin[i];
-    dEK += div_any((m0 + dmom) * (m0 + dmom) - m0 * m0, 2.0 * rho);
+    work[i] = (m0 + dmom) * (m0 + dmom) - m0 * m0;
+  }
+  const double rho2 = 2.0 * rho;
+  if (rcp_range(rho2)) {   // one test for the three of them
+    const double r = rcp_cubic(rho2);
+    for (int i = 0; i < 3; ++i) dEK += work[i] * r;
+  } else {
+    for (int i = 0; i < 3; ++i) dEK += work[i] / rho2;
   }
   a.T_out[c] = T1;
   a.dEgas[c] = kv * (T1 - T0) + dEK;
