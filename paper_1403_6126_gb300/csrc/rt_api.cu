@@ -9,6 +9,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "rt.h"
 #include "rt_ctx.h"
 #include "rt_internal.h"
@@ -254,17 +256,40 @@ rt_status fetch(rt_ctx *c, const double *src, double *dst, long long n) {
   return RT_OK;
 }
 
-// Whether a kernel may access the caller's array p (device_ptrs): doubles on an
-// 8-byte boundary in this device's own memory.  Others (another device's,
-// host memory reached through unified addressing) go by copies.
-bool in_place(const rt_ctx *c, const void *p) {
-  if (!c->opt.device_ptrs || (reinterpret_cast<uintptr_t>(p) & 7) != 0) return false;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeDevice && at.device == c->dev;
+// cuPointerGetAttributes through the runtime (the library does not link the driver's);
+// null where the driver has none.
+auto pointer_attributes() {
+  using Fn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+  static const Fn fn = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Fn>(f);
+  }();
+  return fn;
+}
+
+// Whether a kernel may access n doubles of the caller's array p (device_ptrs): on an
+// 8-byte boundary, within one allocation of this device's own memory.  Others
+// (another device's, host memory reached through unified addressing, an array
+// shorter than the call needs) go by copies, which check their ranges on the host
+// and refuse where a kernel would fault.
+bool in_place(const rt_ctx *c, const void *p, long long n) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+  if (!c->opt.device_ptrs || (at & 7) != 0) return false;
+  const auto attributes = pointer_attributes();
+  unsigned long long type = 0, managed = 0, start = 0, size = 0;   // of whatever width
+  int dev = -1;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void *out[] = {&type, &managed, &dev, &start, &size};
+  if (!attributes || attributes(5, what, out, (CUdeviceptr)at) != CUDA_SUCCESS) return false;
+  return type == CU_MEMORYTYPE_DEVICE && !managed && dev == c->dev && at >= start && at - start <= size &&
+         size - (at - start) >= (unsigned long long)n * sizeof(double);
 }
 
 // Queues the copy of n doubles from the device buffer src to the caller;
@@ -291,7 +316,7 @@ rt_status deliver_fields(rt_ctx *c, const rtg::FieldsOut &want) {
   for (int i = 0; i < 3; ++i) {
     if (!f.dst[i]) f.n[i] = 0;
     count += f.dst[i] != nullptr;
-    direct = direct && (!f.dst[i] || in_place(c, f.dst[i]));
+    direct = direct && (!f.dst[i] || in_place(c, f.dst[i], f.n[i]));
   }
   if (direct && count > 1) {
     RT_CUDA(rtg::launch_fields_out(f, c->stream));
@@ -596,7 +621,7 @@ rt_status rt_set_material(rt_ctx *c, const double *rho, const double *T, const d
   rt_status st;
   // scan: bit 0 = a value out of range or non-finite, bit 1 = some v != 0
   RT_CUDA(cudaMemsetAsync(c->flags + 1, 0, sizeof(int), c->stream));
-  if (in_place(c, rho) && in_place(c, T) && in_place(c, v) && in_place(c, sa) && in_place(c, ss)) {
+  if (in_place(c, rho, N) && in_place(c, T, N) && in_place(c, v, 3 * N) && in_place(c, sa, N) && in_place(c, ss, N)) {
     // one pass stages and scans device arrays that a kernel may read (gas loop of
     // 96 x 80 x 72 cells x 24 angles 233 us, with five copies and a scan 257)
     RT_CUDA(rtg::launch_fields_stage({rho, T, v, sa, ss}, N, c->stage, c->flags + 1, c->stream));
@@ -1196,7 +1221,7 @@ rt_status rt_get_intensity(rt_ctx *c, double *I) {
   if (!c->intensity_set) return fail(RT_E_STATE, "rt_get_intensity: no intensity yet");
   long long total = (long long)c->M * c->N, chunk = c->stage_len;
   if (c->fp64) return deliver(c, (const double *)c->I[c->cur], I, total);
-  if (c->quad && in_place(c, I)) {
+  if (c->quad && in_place(c, I, total)) {
     rtg::AngleMap order{};
     for (int i = 0; i < c->M; ++i) order.slot[i] = (unsigned char)c->order[i];
     RT_CUDA(rtg::launch_intensity_out((const float *)c->I[c->cur], I, c->M, c->N, order, c->stream));
