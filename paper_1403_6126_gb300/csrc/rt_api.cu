@@ -155,12 +155,27 @@ static size_t stage_bytes(long long N, int M, size_t rs, int sides) {
   return std::max(used, sizeof(double) * (size_t)std::max<long long>(10 * N, (long long)8 * M));
 }
 
+// A context's device arrays: N cells, M angles, reals of rs bytes, intensity
+// buffers of I_bytes each, alpha for `sides` distinct cell sides; the float
+// step's (quad) cell centers, the bf16 storage's scratch for Q_m.
+struct ArrayBytes {
+  size_t I, mom, cell, v, T, dMom, ang, inflow, flags, stage, qscr, cen;
+  ArrayBytes(long long N, int M, size_t rs, size_t I_bytes, int sides, bool quad, bool bf16)
+      : I(I_bytes), mom(8 * 10 * (size_t)N), cell(rs * N), v(3 * rs * N), T(8 * (size_t)N), dMom(8 * 3 * (size_t)N),
+        ang(rs * 4 * M), inflow(rs * 6 * M), flags(2 * sizeof(int)), stage(stage_bytes(N, M, rs, sides)),
+        qscr(bf16 ? sizeof(float) * M * (size_t)N : 0), cen(quad ? sizeof(float) * N : 0) {}
+  // What an array of b bytes takes of the context's one allocation.
+  static size_t place(size_t b) { return (b + 511) / 512 * 512; }
+  size_t total() const {
+    return 2 * (place(I) + place(mom) + place(cen) + place(T)) + 3 * place(cell) + place(v) + place(dMom) + place(ang) +
+           place(inflow) + place(flags) + place(stage) + place(qscr);
+  }
+};
+
 size_t rtg::context_bytes(long long N, int M, bool fp64) {
-  const size_t rs = fp64 ? 8 : 4, Nz = (size_t)N, Mz = (size_t)M;
-  const size_t Ms = fp64 ? Mz : 4 * (size_t)((M + 3) / 4);   // stored angles (float: quad padding)
-  const size_t stage = stage_bytes(N, M, rs, 3);
-  const size_t centers = fp64 ? 0 : 2 * sizeof(float) * Nz;   // the float step's cell centers
-  return rs * (2 * Ms * Nz + 6 * Nz + 10 * Mz) + 8 * (2 * 10 * Nz + 3 * Nz) + 16 * Nz + 2 * sizeof(int) + stage + centers;
+  const size_t angles = fp64 ? (size_t)M : 4 * (size_t)((M + 3) / 4);   // stored (float: quad padding)
+  const size_t rs = fp64 ? 8 : 4;
+  return ArrayBytes(N, M, rs, rs * angles * N, 3, !fp64, false).total();
 }
 
 cudaError_t rtg::launch_ctx_step_on(rt_ctx *c, const StepArgs<double> &a, bool vel, TileShape t, cudaStream_t s) {
@@ -548,32 +563,24 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
       if ((float)c->dx[k] == (float)c->dx[d] && (!c->fp64 || c->dx[k] == c->dx[d])) side_of[d] = side_of[k];
     if (d < c->dim && side_of[d] == sides) ++sides;
   }
-  const size_t Nz = (size_t)N, Mz = (size_t)M;
+  const ArrayBytes b(N, M, rs, c->I_bytes, sides, c->quad, c->bf16);
   struct {
     void **p;
     size_t bytes;
   } allocs[] = {
-      {&c->I[0], c->I_bytes},        {&c->I[1], c->I_bytes},        {(void **)&c->mom[0], 8 * 10 * Nz},
-      {(void **)&c->mom[1], 8 * 10 * Nz}, {&c->rho, rs * Nz},       {&c->sa, rs * Nz},
-      {&c->ss, rs * Nz},         {&c->v, rs * 3 * Nz},             {(void **)&c->T, 8 * Nz},
-      {(void **)&c->dEgas, 8 * Nz}, {(void **)&c->dMom, 8 * 3 * Nz}, {&c->ang, rs * 4 * Mz},
-      {&c->inflow, rs * 6 * Mz}, {(void **)&c->flags, 2 * sizeof(int)},
-      {(void **)&c->stage, stage_bytes(N, M, rs, sides)},
-      {(void **)&c->qscr, c->bf16 ? sizeof(float) * Mz * Nz : 0},
-      {(void **)&c->cen[0], c->quad ? sizeof(float) * Nz : 0},
-      {(void **)&c->cen[1], c->quad ? sizeof(float) * Nz : 0},
+      {&c->I[0], b.I},           {&c->I[1], b.I},          {(void **)&c->mom[0], b.mom},
+      {(void **)&c->mom[1], b.mom}, {&c->rho, b.cell},     {&c->sa, b.cell},
+      {&c->ss, b.cell},          {&c->v, b.v},             {(void **)&c->T, b.T},
+      {(void **)&c->dEgas, b.T}, {(void **)&c->dMom, b.dMom}, {&c->ang, b.ang},
+      {&c->inflow, b.inflow},    {(void **)&c->flags, b.flags}, {(void **)&c->stage, b.stage},
+      {(void **)&c->qscr, b.qscr}, {(void **)&c->cen[0], b.cen}, {(void **)&c->cen[1], b.cen},
   };
   // One device allocation for all of them: 15 calls of cudaMalloc and cudaFree
   // cost a burst of short solves a tenth of its time (eight requests 11.0 -> 9.7 ms).
-  size_t total = 0;
   bool fails = false;
-  auto place = [](size_t b) { return (b + 511) / 512 * 512; };
-  for (auto &a : allocs) {
-    if (a.bytes == 0) continue;
-    if ((fails = rtg::allocation_fails())) break;   // each counts for rt_fault_inject
-    total += place(a.bytes);
-  }
-  if (fails || cudaMalloc(&c->block, total) != cudaSuccess) {
+  for (auto &a : allocs)
+    if (a.bytes != 0 && (fails = rtg::allocation_fails())) break;   // each counts for rt_fault_inject
+  if (fails || cudaMalloc(&c->block, b.total()) != cudaSuccess) {
     cudaGetLastError();
     c->block = nullptr;
     free_all(c);
@@ -584,10 +591,10 @@ rt_status rt_create(const rt_grid *g, const rt_angles *ang, double Crat, double 
   for (auto &a : allocs) {
     if (a.bytes == 0) continue;
     *a.p = static_cast<char *>(c->block) + at;
-    at += place(a.bytes);
+    at += ArrayBytes::place(a.bytes);
   }
   if (c->fp64 || (c->sym && c->dim == 3))   // the kernels that read it
-    for (int d = 0; d < c->dim; ++d) c->alpha[d] = (char *)(c->stage + c->stage_len) + rs * Nz * side_of[d];
+    for (int d = 0; d < c->dim; ++d) c->alpha[d] = (char *)(c->stage + c->stage_len) + b.cell * side_of[d];
   // angle table [M][4] = (n_x, n_y, n_z, W) and zero inflow, via the stage
   std::vector<double> tab(4 * (size_t)M);
   for (int i = 0; i < M; ++i) {

@@ -88,7 +88,8 @@ rt_status set_error(rt_status s, const std::string &msg);
 // RT_OK, or RT_E_INVALID (message prefixed by `where`) when the Newton
 // options of o are out of range.
 rt_status check_newton_options(const rt_options &o, const char *where);
-// Device bytes rt_create allocates for N cells and M angles.
+// Device bytes rt_create allocates for N cells and M angles, at most (cells of three
+// different sides).
 size_t context_bytes(long long N, int M, bool fp64);
 // Launch of the fused step for context c (its host tables feed the float
 // kernel's launch-parameter table).
