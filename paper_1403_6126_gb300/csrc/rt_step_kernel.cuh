@@ -16,7 +16,8 @@ constexpr int kHalo = 2;
 
 // Index checking.  A debug build defines RT_BOUNDS_CHECK: every shared- and
 // global-memory index of the float step's per-tile code then passes through
-// RT_IDX(i, n), and an index outside [0, n) adds one to the step's failure
+// RT_IDX(i, n), or RT_AT for pointers, or is one that did (a staged cell, the own
+// cell), and an index outside [0, n) adds one to the step's failure
 // count (the same word as a failed temperature solve, so rt_sync reports
 // it) and is replaced by 0, which turns an out-of-bounds access into a
 // reported error instead of a fault.  In the product build RT_IDX(i, n) is
@@ -26,10 +27,18 @@ __device__ __forceinline__ long long checked_index(long long i, long long n, int
   atomicAdd(status, 1);
   return 0;
 }
+// RT_AT(p, base, n): the same for a pointer that walks through the n elements at
+// base; it is replaced by base.
+template <class T>
+__device__ __forceinline__ T *checked_pointer(T *p, T *base, long long n, int *status) {
+  return base + checked_index(p - base, n, status);
+}
 #ifdef RT_BOUNDS_CHECK
 #define RT_IDX(i, n) (::rtg::stepk::checked_index((i), (n), a.status))
+#define RT_AT(p, base, n) (::rtg::stepk::checked_pointer((p), (base), (n), a.status))
 #else
 #define RT_IDX(i, n) (i)
+#define RT_AT(p, base, n) (p)
 #endif
 constexpr double kPi = 3.14159265358979323846;
 

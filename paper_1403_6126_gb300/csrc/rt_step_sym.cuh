@@ -416,29 +416,29 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
     if constexpr (TAB_PARAM)
       x = tab->e[q][j >> 1];
     else
-      x = reinterpret_cast<const float4 *>(s_tab)[kSymTab / 2 * q + (j >> 1)];
+      x = reinterpret_cast<const float4 *>(s_tab)[RT_IDX(kSymTab / 2 * q + (j >> 1), kSymQuads * kSymTab / 2)];
     return j & 1 ? hi2(x) : lo2(x);
   };
   auto inflow = [&](int face, int m) -> float {
     if constexpr (TAB_PARAM)
       return tab->inflow[face][m];
     else
-      return a.inflow[face * a.M + m];
+      return a.inflow[RT_IDX(face * a.M + m, 6 * a.M)];
   };
   // a cell's quad q: of I^n in whatever order (its smallest value is all that is
   // asked of it), of I_out in stored order (GATHER: until the last write)
   auto load4 = [&](const float *I, int q, long long cell) -> float4 {
-    return reinterpret_cast<const float4 *>(I)[(long long)q * N + cell];
+    return reinterpret_cast<const float4 *>(I)[RT_IDX((long long)q * N + cell, NQ * N)];
   };
   auto store4 = [&](float *I, int q, long long cell, float4 x) {
-    reinterpret_cast<float4 *>(I)[(long long)q * N + cell] = x;
+    reinterpret_cast<float4 *>(I)[RT_IDX((long long)q * N + cell, NQ * N)] = x;
   };
 
   if constexpr (!TAB_PARAM) {
     for (int q = tid; q < NQ; q += NT) {
       float q16[8];
-      for (int i = 0; i < 8; ++i) q16[i] = a.ang[16 * q + i];
-      sym_tab_quad(s_tab + kSymTab * q, q16, a.C, a.dtdx);
+      for (int i = 0; i < 8; ++i) q16[i] = a.ang[RT_IDX(16 * q + i, 4 * a.M)];
+      sym_tab_quad(s_tab + RT_IDX(kSymTab * q, kSymQuads * kSymTab - kSymTab + 1), q16, a.C, a.dtdx);
     }
   }
 
@@ -446,7 +446,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
   const int lx = tid % TX, ly = (tid / TX) % TY, lz = tid / (TX * TY);
   const int gx = org[0] + lx, gy = org[1] + ly, gz = org[2] + lz;
   const bool valid = gx < a.n[0] && gy < a.n[1] && gz < a.n[2];
-  const long long c = valid ? gx + (long long)a.n[0] * (gy + (long long)a.n[1] * gz) : 0;
+  const long long c = valid ? RT_IDX(gx + (long long)a.n[0] * (gy + (long long)a.n[1] * gz), N) : 0;
   float vt[3] = {0, 0, 0}, R = 0, A0 = 1, A1 = 0, a0 = 1, a1 = 0, rd0 = 0, ra0 = 0, scat = 0;
   if (valid) {
     CellIn ci;
@@ -510,7 +510,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s) {
         if (!used(s)) continue;
-        float4 *dst = s_I + (b * ROUND + k) * NBOX + (sl_box[s] & 0xffff);
+        float4 *dst = s_I + RT_IDX((b * ROUND + k) * NBOX + (sl_box[s] & 0xffff), 2 * ROUND * NBOX);
         if constexpr (GATHER) {
           // a cell's place in a plane is a 32-bit byte offset (fewer than 2^28 cells)
           const unsigned at = 16u * (unsigned)sl_g[s];
@@ -520,14 +520,15 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
             return reinterpret_cast<const char *>(a.I_in) + 16 * (long long)(m[h] >> 2) * N + 4 * (m[h] & 3);
           };
           if (tab->pairs[j0 + k]) {
-            copy_async<8>(d, from(0) + at);
-            copy_async<8>(d + 2, from(2) + at);
+            copy_async<8>(d, RT_AT(from(0) + at, reinterpret_cast<const char *>(a.I_in), 16 * NQ * N - 7));
+            copy_async<8>(d + 2, RT_AT(from(2) + at, reinterpret_cast<const char *>(a.I_in), 16 * NQ * N - 7));
           } else {
 #pragma unroll
-            for (int h = 0; h < 4; ++h) copy_async<4>(d + h, from(h) + at);
+            for (int h = 0; h < 4; ++h)
+              copy_async<4>(d + h, RT_AT(from(h) + at, reinterpret_cast<const char *>(a.I_in), 16 * NQ * N - 3));
           }
         } else {
-          copy_async<16>(dst, reinterpret_cast<const float4 *>(a.I_in) + (long long)(j0 + k) * N + sl_g[s]);
+          copy_async<16>(dst, reinterpret_cast<const float4 *>(a.I_in) + RT_IDX((long long)(j0 + k) * N + sl_g[s], NQ * N));
         }
       }
     }
@@ -566,17 +567,17 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
     for (int s = 0; s < SLOTS; ++s) {
       if (!used(s)) continue;
       const int box = sl_box[s] & 0xffff;
-      c_al[box] = KEPT ? al[s][0] : alpha_of(a.dx[0], st[s]);
+      c_al[RT_IDX(box, NBOX)] = KEPT ? al[s][0] : alpha_of(a.dx[0], st[s]);
       if (!same_dx) {   // cells of unequal sides: one alpha per axis
-        c_al[NBOX + box] = KEPT ? al[s][1] : alpha_of(a.dx[1], st[s]);
-        if (DIM == 3) c_al[2 * NBOX + box] = KEPT ? al[s][2] : alpha_of(a.dx[2], st[s]);
+        c_al[RT_IDX(NBOX + box, 3 * NBOX)] = KEPT ? al[s][1] : alpha_of(a.dx[1], st[s]);
+        if (DIM == 3) c_al[RT_IDX(2 * NBOX + box, 3 * NBOX)] = KEPT ? al[s][2] : alpha_of(a.dx[2], st[s]);
       }
       if (VEL) {
         const float w3 = float(3.0 / (4.0 * kPi)) * d2f_rn(E[s]);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          if (d < DIM) c_v[d * NBOX + box] = v[s][d];
-          s_w[d * NBOX + box] = w3 * v[s][d];
+          if (d < DIM) c_v[RT_IDX(d * NBOX + box, 3 * NBOX)] = v[s][d];
+          s_w[RT_IDX(d * NBOX + box, 3 * NBOX)] = w3 * v[s][d];
         }
       }
     }
@@ -588,7 +589,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
   if (tid < G::LINES) {
     Line ln{};
     const int d = G::line(tid, ln), L = d == 0 ? G::LX : d == 1 ? G::LY : G::LZ;
-    s_line[tid].pack(ln);
+    s_line[RT_IDX(tid, G::LINES)].pack(ln);
     const int np = d == 0 ? G::NPX : d == 1 ? G::NPY : G::NPZ;
     float2 *fc = s_fc + (d == 0 ? tid : d == 1 ? G::CY + tid - G::NPX : G::CZ + tid - G::NPX - G::NPY);
     const float *l_al = c_al + (same_dx ? 0 : d * NBOX), *l_v = c_v + d * NBOX;
@@ -607,7 +608,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
         special |= vf == 0.0f;
         v = v1;
       }
-      fc[RT_IDX(f * np, G::NC)] = k;
+      *RT_AT(fc + f * np, s_fc, G::NC) = k;
       al = al1;
     }
   }
@@ -643,23 +644,23 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
         const int box = sl_box[s] & 0xffff, code = sl_box[s] >> 16;
         f2 w0, w1, w2;
         if (VEL) {
-          w0 = dup(s_w[box]);
-          w1 = dup(s_w[NBOX + box]);
-          w2 = dup(s_w[2 * NBOX + box]);
+          w0 = dup(s_w[RT_IDX(box, 3 * NBOX)]);
+          w1 = dup(s_w[RT_IDX(NBOX + box, 3 * NBOX)]);
+          w2 = dup(s_w[RT_IDX(2 * NBOX + box, 3 * NBOX)]);
         }
 #pragma unroll
         for (int k = 0; k < ROUND; ++k) {
           const int j = j0 + k;
           if (j >= NQ) break;
           if (VEL)
-            s_IV[k * NBOX + box] = p_fma(tabv(j, kSymN + 2), w2, p_fma(tabv(j, kSymN), w0, p_mul(tabv(j, kSymN + 1), w1)));
+            s_IV[RT_IDX(k * NBOX + box, ROUND * NBOX)] = p_fma(tabv(j, kSymN + 2), w2, p_fma(tabv(j, kSymN), w0, p_mul(tabv(j, kSymN + 1), w1)));
           if (general && code) {
             // beyond a vacuum or inflow face, the rays that come in: n with mu >
             // 0 through a lower face, mu < 0 through an upper one
             const int ax = (code >> 2) & 3, side = (code >> 4) & 1, face = ax * 2 + side;
             const f2 mu = tabv(j, kSymN + ax);
             const bool infl = (code & 2) != 0;
-            float4 *x = s_I + (b * ROUND + k) * NBOX + box;
+            float4 *x = s_I + RT_IDX((b * ROUND + k) * NBOX + box, 2 * ROUND * NBOX);
             if (side ? (mu.x < 0.0f) : (mu.x > 0.0f)) x->x = infl ? inflow(face, 4 * j) : 0.0f;
             if (side ? (mu.y < 0.0f) : (mu.y > 0.0f)) x->y = infl ? inflow(face, 4 * j + 1) : 0.0f;
             if (side ? (mu.x > 0.0f) : (mu.x < 0.0f)) x->z = infl ? inflow(face, 4 * j + 2) : 0.0f;
@@ -676,7 +677,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
       float4 *F = s_F + kq * G::NF;
       const f2 hc = tabv(j0 + kq, kSymHc + 2 * axis), mud = tabv(j0 + kq, kSymHc + 2 * axis + 1);
       const f2 hca = make_float2(fabsf(hc.x), fabsf(hc.y));
-      const Line at = s_line[line].unpack();
+      const Line at = s_line[RT_IDX(line, G::LINES)].unpack();
       // a walk of L cells; np lines of its kind, F's step sf
       auto walk = [&](auto length, auto gen, auto lines, auto step, float4 *Fl, const float2 *fc) {
         constexpr int L = decltype(length)::value, NP = decltype(lines)::value, SF = decltype(step)::value;
@@ -686,10 +687,10 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
         };
         Walk<VEL, decltype(gen)::value> w;
         f2 va, vb, vc;
-        const float4 ca = cell(In + RT_IDX(at.lo, NBOX), IV + at.lo, &va);
-        const float4 cb = cell(In + RT_IDX(at.lo + at.slo, NBOX), IV + at.lo + at.slo, &vb);
+        const float4 ca = cell(In + RT_IDX(at.lo, NBOX), IV + RT_IDX(at.lo, NBOX), &va);
+        const float4 cb = cell(In + RT_IDX(at.lo + at.slo, NBOX), IV + RT_IDX(at.lo + at.slo, NBOX), &vb);
         const float4 *x = In + RT_IDX(at.core, NBOX);
-        const f2 *v = IV + at.core;
+        const f2 *v = IV + RT_IDX(at.core, NBOX);
         w.start(ca, cb, cell(x, v, &vc), va, vb, vc);
         w.fp = w.fn = dup(0.0f);
 #pragma unroll
@@ -705,11 +706,12 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
             x += at.shi;
             v += at.shi;
           }
-          (void)RT_IDX(x - In, NBOX);
+          x = RT_AT(x, In, NBOX);
+          if (VEL) v = RT_AT(v, IV, NBOX);
           f2 iv;
           const float4 xt = cell(x, v, &iv);
-          const float4 dF = w.face(xt, iv, hc, hca, mud, fc[f * NP]);
-          if (f > 0) Fl[(f - 1) * SF] = dF;
+          const float4 dF = w.face(xt, iv, hc, hca, mud, *RT_AT(fc + f * NP, static_cast<const float2 *>(s_fc), G::NC));
+          if (f > 0) *RT_AT(Fl + (f - 1) * SF, F, G::NF) = dF;
         }
       };
       // one copy of the code per kind of line and for tiles with the two
@@ -742,11 +744,11 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
       const int j = j0 + k;
       if (j >= NQ) break;
       const float4 *F = s_F + k * G::NF;
-      const float4 i4 = s_I[(b * ROUND + k) * NBOX + lx + kHalo + G::RX * (ly + TY * lz)];
-      const float4 fx = F[G::part_x(lx, ly, lz)], fy = F[G::part_y(lx, ly, lz)];
+      const float4 i4 = s_I[RT_IDX((b * ROUND + k) * NBOX + lx + kHalo + G::RX * (ly + TY * lz), 2 * ROUND * NBOX)];
+      const float4 fx = F[RT_IDX(G::part_x(lx, ly, lz), G::NF)], fy = F[RT_IDX(G::part_y(lx, ly, lz), G::NF)];
       f2 dFp = p_add(lo2(fx), lo2(fy)), dFm = p_add(hi2(fx), hi2(fy));
       if (DIM == 3) {
-        const float4 fz = F[G::part_z(lx, ly, lz)];
+        const float4 fz = F[RT_IDX(G::part_z(lx, ly, lz), G::NF)];
         dFp = p_add(dFp, lo2(fz));
         dFm = p_add(dFm, hi2(fz));
       }
@@ -876,12 +878,12 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
         float *out = reinterpret_cast<float *>(s_out + tid);
         auto put = [&](int h, float x) {
           const int m = tab->slot[4 * j + h];
-          out[(m >> 2) * 4 * NT + (m & 3)] = x;
+          out[RT_IDX((m >> 2) * 4 * NT + (m & 3), 4 * (NQ * NT - tid))] = x;
         };
         if (tab->pairs[j]) {   // half the bank conflicts of four words
           auto put2 = [&](int h, f2 x) {
             const int m = tab->slot[4 * j + h];
-            *reinterpret_cast<float2 *>(out + (m >> 2) * 4 * NT + (m & 3)) = x;
+            *reinterpret_cast<float2 *>(RT_AT(out + (m >> 2) * 4 * NT + (m & 3), out, 4 * (NQ * NT - tid) - 1)) = x;
           };
           put2(0, Ip);
           put2(2, Im);
@@ -905,7 +907,7 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
     }
   }
   if constexpr (GATHER)
-    for (int j = 0; j < NQ; ++j) store4(a.I_out, j, c, s_out[j * NT + tid]);
+    for (int j = 0; j < NQ; ++j) store4(a.I_out, j, c, s_out[RT_IDX(j * NT + tid, NQ * NT)]);
   store_cell(a, ci, x, c, mE, mF, mP, pre0, pre1, pre2, cnext);
 }
 
