@@ -880,19 +880,10 @@ __device__ __forceinline__ void process_tile_sym(const StepArgs<float> &a, const
           const int m = tab->slot[4 * j + h];
           out[RT_IDX((m >> 2) * 4 * NT + (m & 3), 4 * (NQ * NT - tid))] = x;
         };
-        if (tab->pairs[j]) {   // half the bank conflicts of four words
-          auto put2 = [&](int h, f2 x) {
-            const int m = tab->slot[4 * j + h];
-            *reinterpret_cast<float2 *>(RT_AT(out + (m >> 2) * 4 * NT + (m & 3), out, 4 * (NQ * NT - tid) - 1)) = x;
-          };
-          put2(0, Ip);
-          put2(2, Im);
-        } else {
-          put(0, Ip.x);
-          put(1, Ip.y);
-          put(2, Im.x);
-          put(3, Im.y);
-        }
+        put(0, Ip.x);
+        put(1, Ip.y);
+        put(2, Im.x);
+        put(3, Im.y);
       } else {
         store4(a.I_out, j, c, mk4(Ip, Im));
       }
