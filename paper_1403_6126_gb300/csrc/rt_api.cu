@@ -710,16 +710,16 @@ rt_status rt_set_intensity(rt_ctx *c, const double *I) {
 namespace {
 
 // The float host table and the device table (stored order) from host_inflow.
-// Waits for the stream.
+// Waits for the stream.  (On the stack: nothing here throws.)
 rt_status inflow_tables(rt_ctx *c) {
   const int M = c->M;
-  std::vector<double> in(6 * (size_t)M);
+  double in[6 * rtg::kMaxAngles];
   for (int f = 0; f < 6; ++f)
     for (int i = 0; i < M; ++i) {
       in[(size_t)f * M + i] = c->host_inflow[(size_t)f * M + c->order[i]];
       c->host_inflowf[(size_t)f * M + i] = (float)in[(size_t)f * M + i];
     }
-  RT_CUDA(cudaMemcpyAsync(c->stage, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  RT_CUDA(cudaMemcpyAsync(c->stage, in, 6 * (size_t)M * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   rt_status st = convert_in(c, c->stage, c->inflow, 6 * M);
   if (st != RT_OK) return st;
   RT_CUDA(cudaStreamSynchronize(c->stream));
