@@ -176,9 +176,11 @@ rt_status rt_set_inflow(rt_ctx *ctx, int axis, int side, const double *I_ghost);
 
 /* Tile of cells one CTA of the step kernel owns (tx x ty x tz, one thread
  * per cell, four in the 32-cell 1-D double tile; ty = 1 for 1-D, tz = 1 below
- * 3-D).  (0, 0, 0) restores the default choice, which follows the grid size.  RT_E_INVALID when the shape is not one of the compiled
- * shapes or exceeds the 227 KB of shared memory (which grows with the angle
- * count).  Float results do not depend on the tile (bitwise); double
+ * 3-D).  (0, 0, 0) restores the default choice, which follows the grid size.
+ * RT_E_INVALID when the shape is not one of the compiled shapes or is not
+ * offered at this angle count: for float, when the tile of a general angle set
+ * exceeds 227 KB of shared memory; for double, when a value per cell and angle
+ * beside the staging arrays would.  Float results do not depend on the tile (bitwise); double
  * results may differ by rounding, as the compiler fuses multiply-adds
  * differently per tile shape and the 32-cell 1-D tile adds its angles up in
  * groups.  The paper has no counterpart (its code runs

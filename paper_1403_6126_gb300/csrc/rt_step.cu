@@ -26,9 +26,10 @@ int shape_list(int dim, TileShape *out) {
   return n;
 }
 
-// Shared memory of a shape within the opt-in limit: the quad kernel for
-// float (its pair table in the launch parameters up to 80 angles), the
-// scalar kernel for double.
+// Whether a shape may be chosen: the quad kernel's shared memory within the
+// opt-in limit for float (its pair table in the launch parameters up to 80
+// angles); for double that of a kernel that kept every right-hand side there
+// (stepk::smem_bytes), which the present one needs far less than.
 template <typename Real>
 bool fits(int dim, int M, bool has_v, TileShape t) {
   const size_t sm = sizeof(Real) == 4

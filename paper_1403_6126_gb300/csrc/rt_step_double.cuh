@@ -25,7 +25,7 @@
 // slab of 8 angles 72 -> 40 us per step, 256 x 128 x 80 shadow problem 577 -> 377
 // us, 40^3 x 24 moving box 1008 -> 689 us.  Since then, with smaller tiles on small
 // grids, alpha formed with the fields, no solves that vanish without velocity and
-// the groups below: slab 11.6, shadow problem 371.
+// the groups below: slab 11.4, shadow problem 371.
 //
 // Reduction used (both implicit steps are linear in I for fixed T):
 //   Step 4 row m:  d_m I_m = r_m + e_m theta - kappa S,   theta = T^4/(4 pi)
@@ -58,7 +58,7 @@ constexpr int kTabD = 19;
 // scheduler), so a small grid gains by more and shorter warps alone: the 1-D tile
 // of 32 cells runs four groups, a warp per scheduler, on lines of two cells.  us
 // per step on 64-cell tiles of one group and here: 512 cells x 8 angles 24.7 and
-// 16.5, 512 x 32 68 and 31, 4096 x 48 99 and 43 (one launch at a time; 11.6 in a
+// 16.5, 512 x 32 68 and 31, 4096 x 48 99 and 43 (one launch at a time; 11.4 in a
 // graph for the first).
 template <int DIM, int TX, int TY, int TZ>
 constexpr int kGroupsD = DIM == 1 && TX == 32 ? 4 : 1;

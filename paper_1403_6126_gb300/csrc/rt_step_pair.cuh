@@ -10,7 +10,8 @@
 // dummy angle (n = 0, W = 0): it adds nothing to any angle sum and is never
 // stored.
 //
-// Three further differences from the scalar kernel:
+// Three further differences from a kernel of one angle per thread with Q_m in
+// shared memory:
 //  * The implicit steps divide in increment form: (r' - s1 - c s2)/a' as
 //    r' - ((a' - 1) r' + s1 + c s2)/a' always, and r/d as r - (d - 1) r/d
 //    where dt C sa < 1, with d - 1 and a' - 1 formed as dt sigma (C - vn)

@@ -19,8 +19,8 @@
 //    cells of the tile along one axis for one quad and walks it with the van
 //    Leer differences, slopes and the last flux in registers: each is formed
 //    once per line (plus its two extension cells), and only I^n, IV and Delta F
-//    per axis pass through shared memory: per cell and quad about 24 128-bit
-//    accesses instead of 48, and two CTA barriers per round of ROUND quads
+//    per axis pass through shared memory: 24 128-bit accesses per cell and quad
+//    instead of 57 (by the wavefronts counted), and two CTA barriers per round of ROUND quads
 //    instead of three per quad.
 //  * I^n comes in by asynchronous copies, a round of quads ahead, in a second
 //    buffer; I~ = I - IV/C is formed as a walk reads a cell.
@@ -35,9 +35,9 @@
 // What bounds it: issue and latency together.  At 96^3 cells x 80 angles (8x8x4
 // tile, two CTAs of 256 threads at 125 registers) it issues 173 thread
 // instructions per cell-angle (the quad kernel 197) at 57 % of the issue rate
-// (48 %), FMA pipe 42 %, shared-memory wavefronts 24 per cell and quad (48),
-// DRAM 0.80 GB for 0.57 GB of intensities: 0.545 ms against 0.726 ms; 128^3 x
-// 80: 1.26 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
+// (48 %), FMA pipe 42 %, 97 shared-memory wavefronts per warp and quad (227),
+// DRAM 0.80 GB for 0.57 GB of intensities: 0.545 ms against 0.726 ms without the
+// profiler; 128^3 x 80: 1.26 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
 // per SM, with the long x and y lines in one phase and the short z lines in
 // the next (0.77: 12 warps); one pair per thread, two threads per cell, 64
 // registers (0.76: 32 warps, but twice the instructions without the packed
