@@ -314,25 +314,26 @@ __device__ __forceinline__ CellSolve solve_cell(const StepArgs<float> &a, const 
     const float beta = a.P * C * (1.0f - v2 * invC * invC) * sa;
     const float c0 = dt * (float(8.0 * kPi) * a.P * sa * Y0 + float(4.0 * kPi) * beta * Z0);
     const float c1 = dt * (float(8.0 * kPi) * a.P * sa * Y1 + float(4.0 * kPi) * beta * Z1);
-    const float cc = c0 + c1 * dth0, c4 = c1 * float(1.0 / (4.0 * kPi));
+    const float c4 = c1 * float(1.0 / (4.0 * kPi));
     // Newton on D from 0; (T^n + D)^4 - (T^n)^4 = D (4 T^3 + D (6 T^2 + D (4 T
     // + D))) with T = T^n keeps every term of the row the size of D; the
     // stopping tolerance is the caller's (at least 1e-6 in float), then one
-    // more step
-    const float T0f = (float)T0, kvf = (float)kv;
+    // more step.  The quotient is the fast one, whose last bits the next iterate
+    // corrects.  It is 0 for divisors above 2^126, so the row is taken times 1/4,
+    // which is exact (rows so small that it might not be have no such divisors).
+    const float T0f = (float)T0;
     const float t2 = T0f * T0f, p3 = 4.0f * t2 * T0f, p2 = 6.0f * t2, p1 = 4.0f * T0f;
+    const float sc = fabsf(fmaf(c4, p3, (float)kv)) < 0x1p-60f ? 1.0f : 0.25f;
+    const float kvs = sc * (float)kv, c4s = sc * c4, cs = sc * (c0 + c1 * dth0);
     const float rtol = fmaxf((float)a.newton_rtol, 1e-6f);
     const int max_it = a.newton_max_it;
     float d = 0.0f;
     int extra = -1, it;
     for (it = 0; it < max_it; ++it) {
       const float T = T0f + d;
-      const float f = fmaf(kvf, d, fmaf(c4, d * fmaf(d, fmaf(d, p1 + d, p2), p3), cc));
-      const float fp = fmaf(4.0f * c4, T * T * T, kvf);
-      // the fast quotient, whose last bits the next iterate corrects, where it is
-      // defined: divisors of magnitude 2^-126 to 2^126
-      const float m = fabsf(fp);
-      float dn = d - (m >= 0x1p-126f && m <= 0x1p126f ? __fdividef(f, fp) : f / fp);
+      const float f = fmaf(kvs, d, fmaf(c4s, d * fmaf(d, fmaf(d, p1 + d, p2), p3), cs));
+      const float fp = fmaf(4.0f * c4s, T * T * T, kvs);
+      float dn = d - __fdividef(f, fp);
       if (!(T0f + dn > 0.0f)) dn = 0.5f * T - T0f;
       const float step = dn - d;
       d = dn;
