@@ -37,7 +37,7 @@
 // instructions per cell-angle (the quad kernel 197) at 57 % of the issue rate
 // (48 %), FMA pipe 42 %, 97 shared-memory wavefronts per warp and quad (227),
 // DRAM 0.80 GB for 0.57 GB of intensities: 0.545 ms against 0.726 ms without the
-// profiler; 128^3 x 80: 1.26 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
+// profiler; 128^3 x 80: 1.27 against 1.72 ms.  Measured and not kept (96^3): 128-thread CTAs, three
 // per SM, with the long x and y lines in one phase and the short z lines in
 // the next (0.77: 12 warps); one pair per thread, two threads per cell, 64
 // registers (0.76: 32 warps, but twice the instructions without the packed
