@@ -98,29 +98,26 @@ __global__ void fields_out_kernel(const FieldsOut f) {
     dst[i] = src[i];
 }
 
-// The caller's angles 4q .. 4q + 3 of every cell as one float4 plane.
-__global__ void plane_out_kernel(const float *__restrict__ I, float4 *__restrict__ dst, int q, long long N,
-                                 const AngleMap map) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-    float v[4];
+// Quad-interleaved intensities of one order of the angles into another: angle m of
+// the result is angle from.slot[m] of src (a multiple of four angles).  Bound by
+// memory: float4s in and out, each cell's words exchanged in shared memory
+// ([M/4][threads], a thread's own column).
+__global__ void reorder_kernel(const float4 *__restrict__ src, float4 *__restrict__ dst, int M, long long N,
+                               const AngleMap from) {
+  extern __shared__ float4 s_q[];
+  const int NT = blockDim.x, tid = threadIdx.x, NQ = M / 4;
+  const float *s = reinterpret_cast<const float *>(s_q);
+  for (long long c = blockIdx.x * (long long)NT + tid; c < N; c += (long long)gridDim.x * NT) {
+#pragma unroll 4
+    for (int q = 0; q < NQ; ++q) s_q[q * NT + tid] = src[q * N + c];
+    for (int q = 0; q < NQ; ++q) {
+      float v[4];
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const long long k = map.slot[4 * q + h];
-      v[h] = I[(k >> 2) * 4 * N + 4 * c + (k & 3)];
-    }
-    dst[c] = make_float4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-__global__ void plane_in_kernel(const float4 *__restrict__ src, float *__restrict__ I, int q, long long N,
-                                const AngleMap map) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-    const float4 x = src[c];
-    const float v[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const long long k = map.slot[4 * q + h];
-      I[(k >> 2) * 4 * N + 4 * c + (k & 3)] = v[h];
+      for (int h = 0; h < 4; ++h) {
+        const int k = from.slot[4 * q + h];
+        v[h] = s[4 * ((k >> 2) * NT + tid) + (k & 3)];
+      }
+      dst[q * N + c] = make_float4(v[0], v[1], v[2], v[3]);
     }
   }
 }
@@ -319,13 +316,10 @@ cudaError_t launch_fields_out(const FieldsOut &f, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_plane_out(const float *I, float *dst, int q, long long N, const AngleMap &map, cudaStream_t s) {
-  plane_out_kernel<<<grid_for(N, 256), 256, 0, s>>>(I, reinterpret_cast<float4 *>(dst), q, N, map);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_plane_in(const float *src, float *I, int q, long long N, const AngleMap &map, cudaStream_t s) {
-  plane_in_kernel<<<grid_for(N, 256), 256, 0, s>>>(reinterpret_cast<const float4 *>(src), I, q, N, map);
+cudaError_t launch_reorder(const float *src, float *dst, int M, long long N, const AngleMap &from, cudaStream_t s) {
+  constexpr int NT = 128;
+  reorder_kernel<<<grid_for(N, NT), NT, (M / 4) * NT * sizeof(float4), s>>>(
+      reinterpret_cast<const float4 *>(src), reinterpret_cast<float4 *>(dst), M, N, from);
   return cudaGetLastError();
 }
 

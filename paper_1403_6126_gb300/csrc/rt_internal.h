@@ -207,10 +207,9 @@ cudaError_t launch_fields_out(const FieldsOut &f, cudaStream_t s);
 // caller's index of each stored angle).
 cudaError_t launch_intensity_out(const float *src, double *dst, int M, long long N, const AngleMap &order,
                                  cudaStream_t s);
-// One plane of four angles (the caller's 4q .. 4q + 3) of an array stored
-// through map, as float4 per cell: out of I into dst, or (in) from src into I.
-cudaError_t launch_plane_out(const float *I, float *dst, int q, long long N, const AngleMap &map, cudaStream_t s);
-cudaError_t launch_plane_in(const float *src, float *I, int q, long long N, const AngleMap &map, cudaStream_t s);
+// Quad-layout intensities in another order of their angles (a multiple of four, at
+// most 80): angle m of dst is angle from.slot[m] of src.
+cudaError_t launch_reorder(const float *src, float *dst, int M, long long N, const AngleMap &from, cudaStream_t s);
 
 // bf16 storage: encode a float intensity array [M][N] as deviations from
 // the mean intensity of each cell (E [N] its energy density), and decode
