@@ -37,7 +37,7 @@ struct rt_ctx {
   double *mom[2] = {nullptr, nullptr};   // E, F, P [10][N], double for every precision
   int cur = 0;
   void *rho = nullptr, *sa = nullptr, *ss = nullptr, *v = nullptr;
-  void *alpha[3] = {nullptr, nullptr, nullptr};   // per axis [N], behind the staging buffer
+  void *alpha[3] = {nullptr, nullptr, nullptr};   // per axis [N], at the end of the staging buffer
   double *T = nullptr, *dEgas = nullptr;
   double *dMom = nullptr;                 // Delta(rho v) [3][N]
   void *ang = nullptr, *inflow = nullptr;
